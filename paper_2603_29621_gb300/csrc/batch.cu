@@ -3,6 +3,9 @@
 // frozen-data mode).  Each problem's blocks follow the previous problem's; every block reads its
 // problem's fields (vectors, mesh size, physics) from the table, so the arithmetic per cell is the
 // one of a single-problem launch and results are bitwise those of separate applications.
+#include <algorithm>
+
+#include "ns_lines.hpp"
 #include "op_kernel.cuh"
 #include "problem.hpp"
 #include "vec.hpp"
@@ -16,6 +19,7 @@ struct MultiOp {
   std::vector<const void*> src;
   std::vector<void*> dst;
   std::vector<MultiColour> col;
+  NsMulti ns[2];   // uniform 3D stabilised levels: the members on the line and on the plane kernel
   DevBuf probs, pid;
 };
 
@@ -27,8 +31,37 @@ static int64_t colour_cells(const OpLaunch& L, int c) {
   return nc;
 }
 
+static void fill_ns(MultiOp& m, Budget* bud) {
+  std::vector<char> desc;
+  std::vector<int32_t> pid;
+  size_t desc_at[2], pid_at[2];
+  for (int planes = 0; planes < 2; ++planes) {
+    desc_at[planes] = desc.size();
+    pid_at[planes] = pid.size();
+    int members = 0;
+    for (size_t i = 0; i < m.lv.size(); ++i) {
+      const OpLevel& lv = *m.lv[i];
+      if (ns_planes(m.prec, lv.L.lc[m.prec]) != (planes == 1)) continue;
+      const int64_t nb = ns_blocks(lv.L, m.prec);
+      if (pid.size() + (size_t)nb >= (size_t)1 << 31)
+        throw Error(kErrUnsupported, "multi-problem launch: too many blocks");
+      ns_descriptor(lv.L, m.prec, m.src[i], lv.rows[m.prec].get(), (int32_t)(pid.size() - pid_at[planes]), desc);
+      pid.insert(pid.end(), (size_t)nb, members++);
+      m.ns[planes].cmax = std::max(m.ns[planes].cmax, lv.L.lc[m.prec]);
+    }
+    m.ns[planes].blocks = (int64_t)(pid.size() - pid_at[planes]);
+  }
+  m.probs = upload(bud, desc);
+  m.pid = upload(bud, pid);
+  for (int planes = 0; planes < 2; ++planes) {
+    m.ns[planes].probs = m.probs.as<char>() + desc_at[planes];
+    m.ns[planes].block_pid = m.pid.as<int32_t>() + pid_at[planes];
+  }
+}
+
 template <typename T>
 static void fill(MultiOp& m, Budget* bud) {
+  if (m.L0->lq[m.prec]) return fill_ns(m, bud);
   const OpLaunch& L0 = *m.L0;
   const int nmem = (int)m.lv.size();
   const int ncol = L0.n_colors;
@@ -86,7 +119,8 @@ MultiOp* multi_op_create(const std::vector<const OpLevel*>& lv, const std::vecto
   for (const OpLevel* l : lv) {
     const OpLaunch& L = l->L;
     if (!L.structured || L.dim != L0.dim || L.k != L0.k || L.op != L0.op || L.n_colors != L0.n_colors ||
-        (L.fq[prec] != nullptr) != (L0.fq[prec] != nullptr) || L.warps[prec] != L0.warps[prec])
+        (L.fq[prec] != nullptr) != (L0.fq[prec] != nullptr) ||
+        (L.lq[prec] != nullptr) != (L0.lq[prec] != nullptr) || L.warps[prec] != L0.warps[prec])
       throw Error(kErrArg, "multi-op: members differ in kind, degree, layout or block size");
   }
   auto m = std::make_unique<MultiOp>();
@@ -104,6 +138,17 @@ MultiOp* multi_op_create(const std::vector<const OpLevel*>& lv, const std::vecto
 
 // dst_i = A_i src_i for every member (constrained rows dst = src), one launch per colour.
 void multi_vmult(const MultiOp& m, cudaStream_t s) {
+  if (m.ns[0].blocks || m.ns[1].blocks) {
+    for (const NsMulti& part : m.ns)
+      if (part.blocks) ns_cells_multi(*m.L0, m.prec, part, s);
+    for (size_t i = 0; i < m.lv.size(); ++i) {
+      NsAfterArgs a;
+      a.dst = m.dst[i];
+      a.src = m.src[i];
+      ns_nodes(m.lv[i]->L, m.prec, a, m.lv[i]->rows[m.prec].get(), s);
+    }
+    return;
+  }
   const size_t es = m.prec == 0 ? 8 : 4;
   for (size_t i = 0; i < m.lv.size(); ++i) MFNS_CUDA(cudaMemsetAsync(m.dst[i], 0, m.lv[i]->n_dofs * es, s));
   for (int c = 0; c < (int)m.col.size(); ++c) op_apply_multi(*m.L0, m.prec, c, m.col[c], s);

@@ -1,5 +1,6 @@
 // The operator kernel (see op_kernel.cuh for the building blocks).
 #pragma once
+#include "ns_lines.cuh"
 #include "op_kernel.cuh"
 
 namespace mfns {
@@ -52,6 +53,12 @@ template <int DIM, int K, int OP, typename T>
 struct OpMinBlocks {
   static constexpr int value = 1;
 };
+// the diagonal of a uniform 3D stabilised level keeps the frozen state's point values in registers
+// through its unit-vector passes (no staged blocks there): no occupancy bound
+template <int DIM, int K, int OP, typename T, bool DIAG, int FQ>
+constexpr int op_min_blocks() {
+  return DIAG && FQ == 0 ? 1 : OpMinBlocks<DIM, K, OP, T>::value;
+}
 #ifndef MFNS_STABNS_Q2_F32_MINBLOCKS
 #define MFNS_STABNS_Q2_F32_MINBLOCKS 6
 #endif
@@ -130,7 +137,7 @@ template <int DIM, int K, int OP, typename T, bool STRUCT, bool DIAG, int FQ = 0
           bool MULTI = false, bool DEFER = false>
 __global__ void __launch_bounds__(kOpWarps * 32, (EPI && OpMinBlocks<DIM, K, OP, T>::value > 1)
                                                      ? OpMinBlocks<DIM, K, OP, T>::value - 1
-                                                     : OpMinBlocks<DIM, K, OP, T>::value)
+                                                     : op_min_blocks<DIM, K, OP, T, DIAG, FQ>())
 op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
   constexpr int Q = K + 1, N = K + 1, NP = OP == OP_STOKES ? K : K + 1;
   using Tr = OpTraits<OP, DIM>;
@@ -243,7 +250,8 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
   }
   // the next colour's grid may be scheduled once every block of this one has started (it waits
   // for this grid's completion before it touches dst)
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  // (the set-up pass lets nothing start early: its output is read as constant data)
+  if constexpr (FQ != 2) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const T h = STRUCT ? hs : args.hcell[cell];
   const uint32_t mask = STRUCT ? 0u : args.mask[cell];
   // warp-uniform: every team of the warp takes the constraint path if one needs it
@@ -466,7 +474,36 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
       const T a = T(2) * dt_inv_, b2 = T(4) * un2 * inv_h * inv_h, c = T(12) * nu * inv_h * inv_h;
       tau[l] = T(1) / sqrt(a * a + b2 + c * c);
     }
-    if constexpr (FQ == 2) {
+    if constexpr (FQ == 2 && STRUCT && DIM == 3) {
+      // quads (U / h, tau), (G_i, tau Rbar_i / h) with the linearisation factors, as k_ns_cells reads them
+      if (valid) {
+        const uint32_t tcell = (uint32_t)cell, blk = tcell / (uint32_t)args.lc;
+        const int sl = (int)(tcell - blk * (uint32_t)args.lc);
+#pragma unroll
+        for (int l = 0; l < Q; ++l) {
+          T v[4][4];
+#pragma unroll
+          for (int i = 0; i < DIM; ++i) {
+            v[0][i] = Ub[i][l] * inv_h;
+#pragma unroll
+            for (int j = 0; j < DIM; ++j) v[1 + i][j] = cf_[2] * Gb[i][j][l];
+            v[1 + i][3] = cf_[4] * tau[l] * Rb[i][l] * inv_h;
+          }
+          v[0][3] = tau[l];
+#pragma unroll
+          for (int q4 = 0; q4 < 4; ++q4)
+#pragma unroll
+            for (int hf = 0; hf < (int)sizeof(T) / 4; ++hf) {
+              T* fp = args.lq + ns_fq_at<T, Q>(blk, ti + Q * tj, l, q4, hf, sl, args.lc);
+              if constexpr (sizeof(T) == 4)
+                *reinterpret_cast<float4*>(fp) = make_float4(v[q4][0], v[q4][1], v[q4][2], v[q4][3]);
+              else
+                *reinterpret_cast<double2*>(fp) = make_double2(v[q4][2 * hf], v[q4][2 * hf + 1]);
+            }
+        }
+      }
+      return;  // set-up pass: nothing else to do (no __syncwarp follows)
+    } else if constexpr (FQ == 2) {
       if (valid) {
         constexpr int B = FrozenPoint<DIM>::template block<T>(Q);
         T* fp = fqd + (size_t)cellpos * B;

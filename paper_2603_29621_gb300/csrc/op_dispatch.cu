@@ -115,7 +115,7 @@ int64_t frozen_point_values_per_cell(int dim, int k) {
 }
 
 void op_precompute_frozen(const OpLaunch& L, int prec, cudaStream_t s) {
-  if (L.op != OP_STAB_NS || !L.fq[prec]) return;
+  if (L.op != OP_STAB_NS || (!L.fq[prec] && !L.lq[prec])) return;
   if (prec == 0)
     dispatch<double>(L, nullptr, nullptr, false, s, 2);
   else

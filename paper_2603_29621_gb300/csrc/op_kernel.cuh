@@ -87,6 +87,8 @@ struct OpArgs {
   // stabilised NS: frozen quantities at the Gauss points, precomputed (u, grad u, Rbar, tau per
   // point), laid out [cell position][lane][point][NFQ] with cell position = colour offset + index
   T* fq;
+  T* lq;                 // set-up pass on uniform 3D levels: the layout of ns_lines.cuh, lc cells per block
+  int lc;
   int64_t color_offset;  // structured: cells of the colours before this one
   // several right-hand sides in one launch: blockIdx.y selects src/dst + blockIdx.y * col_stride
   // (0 in diagonal mode, where blockIdx.y splits the unit-vector passes instead)

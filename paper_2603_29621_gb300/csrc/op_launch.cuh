@@ -71,6 +71,8 @@ static void fill_common(const OpLaunch& L, OpArgs<T, Q, N, NP>& a) {
   for (int b = 0; b < 7; ++b) a.cf[b] = (L.terms >> b) & 1 ? T(1) : T(0);
   a.err = op_wait_flag();
   a.fq = reinterpret_cast<T*>(L.fq[prec]);
+  a.lq = reinterpret_cast<T*>(L.lq[prec]);
+  a.lc = L.lc[prec];
   a.gexp = reinterpret_cast<const T*>(L.gexp[prec]);
 }
 
@@ -122,19 +124,16 @@ void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t 
     const uint64_t bit = 1ull << (dev & 63);
     if (fq == 1 && !(attr_done.load() & bit)) {
       const int mx = (int)op_smem_bytes<DIM, K, OP, T>(kOpWarps, true);
-      MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
       MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, false, true, 1>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
       MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, false, false, 1>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-      MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-      // the structured product's blocks are one warp with its staged blocks: ask for the largest
-      // shared-memory carveout so that shared memory never caps the resident blocks below the
-      // register limit
-      MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1>,
-                                     cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+      if constexpr (DIM == 2) {  // uniform 3D levels with stored point values: ns_lines.cuh
+        MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1, true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+      }
       attr_done.fetch_or(bit);
     }
   }
@@ -187,11 +186,16 @@ void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t 
         else
           go(op_kernel<DIM, K, OP, T, false, false, 3>, smem);
       } else if (fq == 1) {
-        if (structured && fused)
-          go(op_kernel<DIM, K, OP, T, true, false, 1, true>, smem_fq);
-        else if (structured)
-          go(op_kernel<DIM, K, OP, T, true, false, 1>, smem_fq);
-        else if (diag)
+        if (structured && DIM == 3)
+          throw Error(kErrArg, "stored point values of a uniform 3D level: another layout");
+        if constexpr (DIM == 2) {
+          if (structured && fused)
+            go(op_kernel<DIM, K, OP, T, true, false, 1, true>, smem_fq);
+          else if (structured)
+            go(op_kernel<DIM, K, OP, T, true, false, 1>, smem_fq);
+        }
+        if (structured) {
+        } else if (diag)
           go(op_kernel<DIM, K, OP, T, false, true, 1>, smem_fq);
         else
           go(op_kernel<DIM, K, OP, T, false, false, 1>, smem_fq);
@@ -220,7 +224,7 @@ void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t 
   }
 }
 
-// Deferred product of a uniform 3D stabilised level: one launch over every colour (blockIdx.y =
+// Deferred product of a small uniform 3D level: one launch over every colour (blockIdx.y =
 // colour) writing each cell's contributions to `defer`; k_gather_cells forms dst from them.
 template <int DIM, int K, int OP, typename T>
 void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, cudaStream_t s) {
@@ -246,24 +250,6 @@ void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, cudaStream_t 
       maxc = std::max(maxc, nc);
     }
     const dim3 grid((unsigned)((maxc + cells_per_block - 1) / cells_per_block), 8u);
-    if constexpr (OP == OP_STAB_NS) {
-      if (a.fq) {  // the precomputed frozen point data, staged per cell
-        const size_t sm = op_smem_bytes<DIM, K, OP, T>(warps, true);
-        auto kern = op_kernel<DIM, K, OP, T, true, false, 1, false, false, true>;
-        static std::atomic<uint64_t> attr_done{0};  // per device, for the largest block size
-        int dev = 0;
-        MFNS_CUDA(cudaGetDevice(&dev));
-        const uint64_t bit = 1ull << (dev & 63);
-        if (!(attr_done.load() & bit)) {
-          MFNS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)op_smem_bytes<DIM, K, OP, T>(kOpWarps, true)));
-          attr_done.fetch_or(bit);
-        }
-        kern<<<grid, warps * 32, sm, s>>>(a);
-        MFNS_CUDA(cudaGetLastError());
-        return;
-      }
-    }
     op_kernel<DIM, K, OP, T, true, false, 0, false, false, true>
         <<<grid, warps * 32, op_smem_bytes<DIM, K, OP, T>(warps, false), s>>>(a);
     MFNS_CUDA(cudaGetLastError());
@@ -288,13 +274,13 @@ void op_launch_multi(const OpLaunch& L, int color, const MultiColour& mc, cudaSt
     a.err = op_wait_flag();
     const int warps = L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
     bool staged = false;
-    if constexpr (OP == OP_STAB_NS) staged = L.fq[prec] != nullptr;
+    if constexpr (OP == OP_STAB_NS && DIM == 2) staged = L.fq[prec] != nullptr;
     if (staged) {
       static std::atomic<uint64_t> attr_done{0};
       int dev = 0;
       MFNS_CUDA(cudaGetDevice(&dev));
       const uint64_t bit = 1ull << (dev & 63);
-      if constexpr (OP == OP_STAB_NS) {
+      if constexpr (OP == OP_STAB_NS && DIM == 2) {
         if (!(attr_done.load() & bit)) {
           MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1, false, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -302,7 +288,7 @@ void op_launch_multi(const OpLaunch& L, int color, const MultiColour& mc, cudaSt
           attr_done.fetch_or(bit);
         }
       }
-      if constexpr (OP == OP_STAB_NS)
+      if constexpr (OP == OP_STAB_NS && DIM == 2)
         op_kernel<DIM, K, OP, T, true, false, 1, false, true>
             <<<mc.nblocks, warps * 32, op_smem_bytes<DIM, K, OP, T>(warps, true), s>>>(a);
     } else {

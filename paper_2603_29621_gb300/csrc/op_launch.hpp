@@ -57,6 +57,8 @@ struct OpLaunch {
   std::vector<double> S, Sp, D, D2, W, P, Pp;
   KernelTimer* timer = nullptr;     // optional per-launch timing
   void* fq[2] = {nullptr, nullptr}; // stabilised NS: precomputed frozen point data (fp64 / fp32)
+  void* lq[2] = {nullptr, nullptr}; // ... of a uniform 3D level, in the layout of ns_lines.cuh (fq is then null)
+  int lc[2] = {0, 0};               // cells per block of that layout
   int warps[2] = {0, 0};            // warps per block per precision (0 = not tuned yet: use 4)
   const uint8_t* lastc = nullptr;   // per main node: index of the last colour whose cells touch it
 };
@@ -74,7 +76,7 @@ int autotune_warps(OpLaunch& L, int prec, void* src, void* dst, int64_t n, cudaS
 
 // Stabilised NS: number of precomputed values per cell (lanes x points x values per point).
 int64_t frozen_point_values_per_cell(int dim, int k);
-// Fill L.fq[prec] (device buffer of n_cells * frozen_point_values_per_cell) from the frozen state.
+// Fill L.fq[prec] (device buffer of n_cells * frozen_point_values_per_cell) or L.lq[prec] from the frozen state.
 void op_precompute_frozen(const OpLaunch& L, int prec, cudaStream_t s);
 
 // Stabilised NS: dst = F(frozen state), the nonlinear residual on the free rows (dst zeroed by the

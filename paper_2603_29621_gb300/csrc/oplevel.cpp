@@ -5,6 +5,7 @@
 #include <numeric>
 #include <unordered_map>
 
+#include "ns_lines.hpp"
 #include "problem.hpp"
 #include "vec.hpp"
 
@@ -21,7 +22,7 @@ size_t OpLevel::bytes() const {
   size_t b = fq[0].bytes() + fq[1].bytes() + cell_u.bytes() + cell_p.bytes() + cell_f.bytes() + mask.bytes() + constrained.bytes() +
              hang_dof.bytes() + hang_ptr.bytes() + hang_src.bytes() + pres.bytes() + tnodes.bytes() +
              tpnodes.bytes();
-  for (int i = 0; i < 2; ++i) b += hcell[i].bytes() + frozen[i].bytes() + hang_w[i].bytes() + dinv[i].bytes();
+  for (int i = 0; i < 2; ++i) b += rows[i].bytes() + hcell[i].bytes() + frozen[i].bytes() + hang_w[i].bytes() + dinv[i].bytes();
   return b;
 }
 
@@ -185,7 +186,19 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
     lv.frozen[1] = upload_as<float>(bud, fz);
     L.frozen[0] = lv.frozen[0].get();
     L.frozen[1] = lv.frozen[1].get();
-    if (ph.precompute_frozen) {
+    if (ph.precompute_frozen && ns_lines(L)) {
+      // uniform 3D levels: the layout of ns_lines.cuh, and the rows through which a product is summed
+      for (int prec = 0; prec < 2; ++prec) {
+        L.lc[prec] = ns_cells_per_block(k, prec, (int64_t)nc);
+        lv.fq[prec].alloc(bud, ns_fq_bytes(L, prec));
+        lv.rows[prec].alloc(bud, ns_rows_bytes(L, prec));
+        // spare slots of the last block hold zeros; the tails that no block writes are not read
+        MFNS_CUDA(cudaMemset(lv.fq[prec].get(), 0, ns_fq_bytes(L, prec)));
+        L.lq[prec] = lv.fq[prec].get();
+        op_precompute_frozen(L, prec, 0);
+      }
+      MFNS_CUDA(cudaStreamSynchronize(0));
+    } else if (ph.precompute_frozen) {
       // point values of the frozen state (u, grad u, Rbar, tau), computed once by the cell kernel
       const int64_t per_cell = frozen_point_values_per_cell(dim, k);
       for (int prec = 0; prec < 2; ++prec) {
@@ -253,9 +266,10 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
     for (int32_t i : lv.constrained_host) km[(size_t)i >> 5] |= 1u << (i & 31);
     lv.keep_mask = upload(bud, km);
   }
-  // small uniform 3D stabilised, vector-Laplacian and pressure-mass levels: products as one launch
-  // over all colours plus a gather pass (their eight colour launches are latency, not work)
-  if (lv.L.structured && (op == OP_STAB_NS || op == OP_STOKES_A || op == OP_PMASS) && dim == 3 &&
+  // small uniform 3D stabilised (frozen state recomputed), vector-Laplacian and pressure-mass levels:
+  // products as one launch over all colours plus a gather pass (their eight colour launches are
+  // latency, not work)
+  if (lv.L.structured && !lv.L.lq[0] && (op == OP_STAB_NS || op == OP_STOKES_A || op == OP_PMASS) && dim == 3 &&
       (int64_t)lv.L.n_cells <= kDeferMaxCells) {
     const size_t entries = (size_t)lv.L.n_cells * (size_t)((k + 1) * (k + 1) * (k + 1)) * lv.NU;
     for (int prec = 0; prec < 2; ++prec) lv.defer[prec].alloc(bud, entries * esize(prec));
@@ -272,6 +286,14 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
 
 void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cudaStream_t s) {
   if (lv.hp) return hp_vmult(lv, prec, src, dst, s);
+  if (lv.L.lq[prec]) {
+    NsAfterArgs a;
+    a.dst = dst;
+    a.src = src;
+    ns_cells(lv.L, prec, src, lv.rows[prec].get(), s);
+    ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
+    return;
+  }
   // clearing kernel, then the colour launches (each may start before its predecessor drains);
   // on uniform meshes the clearing kernel also writes the identity rows, which no colour touches
   if (lv.defer[prec].get()) {  // small uniform levels: one launch over all colours, one gather pass
@@ -288,6 +310,33 @@ void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cuda
     vcopy_idx<double>((double*)dst, (const double*)src, lv.constrained.as<int32_t>(), nc, s);
   else
     vcopy_idx<float>((float*)dst, (const float*)src, lv.constrained.as<int32_t>(), nc, s);
+}
+
+bool oplevel_fuses(const OpLevel& lv, int prec) { return lv.L.lq[prec] != nullptr; }
+
+void oplevel_update(const OpLevel& lv, int prec, void* x, void* d, const void* b, const void* dinv, double c1,
+                    double c2, cudaStream_t s) {
+  NsAfterArgs a;
+  a.after = 1;
+  a.dst = x;
+  a.src = x;
+  a.b = b;
+  a.dinv = dinv;
+  a.d = d;
+  a.c1 = c1;
+  a.c2 = c2;
+  ns_cells(lv.L, prec, x, lv.rows[prec].get(), s);
+  ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
+}
+
+void oplevel_residual(const OpLevel& lv, int prec, const void* x, const void* b, void* r, cudaStream_t s) {
+  NsAfterArgs a;
+  a.after = 2;
+  a.dst = r;
+  a.src = x;
+  a.b = b;
+  ns_cells(lv.L, prec, x, lv.rows[prec].get(), s);
+  ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
 }
 
 void oplevel_vmult_cols(const OpLevel& lv, int prec, const void* X, void* Y, int ncols, cudaStream_t s) {

@@ -38,7 +38,8 @@ struct OpLevel {
   std::vector<int32_t> constrained_host;
   DevBuf constrained;                   // identity rows
   DevBuf keep_mask;                     // uniform meshes: bitmask of the identity rows (see oplevel_vmult)
-  DevBuf defer[2];                      // small uniform 3D stabilised levels: per-cell contributions (FP64 / FP32)
+  DevBuf defer[2];                      // small uniform 3D levels: per-cell contributions (FP64 / FP32)
+  DevBuf rows[2];                       // uniform 3D stabilised levels: rows of a product (ns_lines.hpp)
   int64_t n_hang = 0;
   DevBuf hang_dof, hang_ptr, hang_src, hang_w[2];
   std::vector<int32_t> pres_host;
@@ -110,6 +111,12 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
                    bool edge_dirichlet = false);
 void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cudaStream_t s);
 void oplevel_diag(const OpLevel& lv, int prec, void* diag, cudaStream_t s);
+// Levels whose product ends in a node pass that can apply what follows it (x, d, b in place of the
+// separate vector kernels): d = c1 d + c2 dinv (b - A x), x += d;  r = b - A x.
+bool oplevel_fuses(const OpLevel& lv, int prec);
+void oplevel_update(const OpLevel& lv, int prec, void* x, void* d, const void* b, const void* dinv, double c1,
+                    double c2, cudaStream_t s);
+void oplevel_residual(const OpLevel& lv, int prec, const void* x, const void* b, void* r, cudaStream_t s);
 // One smoothing step with the update fused into the operator application (t: scratch):
 // d = c1 d + c2 dinv (b - A x), xout = x + d  (xout must not alias x)
 void oplevel_smooth_step(const OpLevel& lv, int prec, const void* x, void* xout, void* d, const void* b,

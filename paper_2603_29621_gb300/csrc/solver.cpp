@@ -353,6 +353,11 @@ static void level_dinv(Problem& p, OpLevel& lv, cudaStream_t s, bool fp32 = fals
   }
 }
 
+// the block size of the cell kernel; uniform 3D stabilised levels have their own (ns_lines.hpp)
+static void autotune_level(OpLaunch& L, int prec, void* a, void* b, int64_t n, cudaStream_t s) {
+  if (!L.lq[prec]) autotune_warps(L, prec, a, b, n, s);
+}
+
 void autotune(Problem& p, cudaStream_t s) {
   // scratch: the level workspaces (contents are overwritten before any use)
   for (int prec = 0; prec < 2; ++prec)
@@ -363,7 +368,7 @@ void autotune(Problem& p, cudaStream_t s) {
       if (lv.hp) {  // hp levels: every degree group on its own
         for (auto& g : lv.hp->groups) autotune_warps(g->L, prec, w.x.get(), w.t.get(), lv.n_dofs, s);
       } else {
-        autotune_warps(lv.L, prec, w.x.get(), w.t.get(), lv.n_dofs, s);
+        autotune_level(lv.L, prec, w.x.get(), w.t.get(), lv.n_dofs, s);
       }
     }
   if (p.ls) {
@@ -371,8 +376,8 @@ void autotune(Problem& p, cudaStream_t s) {
       for (int prec = 0; prec < 2; ++prec) {
         Workspace& w = lv->ws[prec];
         MFNS_CUDA(cudaMemsetAsync(w.x.get(), 0, lv->op->n_dofs * esize(prec), s));
-        autotune_warps(lv->op->L, prec, w.x.get(), w.t.get(), lv->op->n_dofs, s);
-        autotune_warps(lv->full->L, prec, w.x.get(), w.t.get(), lv->full->n_dofs, s);
+        autotune_level(lv->op->L, prec, w.x.get(), w.t.get(), lv->op->n_dofs, s);
+        autotune_level(lv->full->L, prec, w.x.get(), w.t.get(), lv->full->n_dofs, s);
       }
     autotune(*p.ls->base, s);
   }
@@ -386,7 +391,7 @@ void autotune(Problem& p, cudaStream_t s) {
       if (lv->hp) {  // hp operators: every degree group on its own (the level's own launch is empty)
         for (auto& g : lv->hp->groups) autotune_warps(g->L, prec, a, b, lv->n_dofs, s);
       } else {
-        autotune_warps(lv->L, prec, a, b, lv->n_dofs, s);
+        autotune_level(lv->L, prec, a, b, lv->n_dofs, s);
       }
     }
   }
@@ -608,9 +613,11 @@ static void smooth_op(const Problem& p, OpLevel& lv, Workspace& w, int prec, con
   // into the cell kernel's last-colour scatter; the new iterate then goes to the other of two
   // buffers (x and the level's residual vector, free while smoothing).  Otherwise the product
   // is written out and a streaming kernel applies the update.
-  const bool fused = p.fused_smoother && lv.L.structured && lv.L.lastc;
+  const bool nodes = oplevel_fuses(lv, prec);  // the product's node pass applies the update
+  const bool fused = p.fused_smoother && lv.L.structured && lv.L.lastc && !nodes;
   T* cur = x;
   auto step = [&](double c1, double c2) {
+    if (nodes) return oplevel_update(lv, prec, x, d, b, dinv, (double)(T)c1, (double)(T)c2, s);
     if (!fused) {
       oplevel_vmult(lv, prec, x, t, s);
       vcheby<T>(x, d, b, t, dinv, (T)c1, (T)c2, n, s);
@@ -702,7 +709,9 @@ static void vcycle_level(Problem& p, int prec, int l, const T* b, T* x, cudaStre
   Workspace& wc = p.ws[prec][l + 1];
   const int64_t n = lv.n_dofs;
   smooth_t<T>(p, l, prec, b, x, true, p.smoother_degree, s);
-  if (p.fused_smoother && lv.L.structured && lv.L.lastc) {
+  if (oplevel_fuses(lv, prec)) {
+    oplevel_residual(lv, prec, x, b, w.r.get(), s);
+  } else if (p.fused_smoother && lv.L.structured && lv.L.lastc) {
     oplevel_residual_fused(lv, prec, x, b, w.r.get(), w.t.get(), s);  // r = b - A x, fused
   } else {
     oplevel_vmult(lv, prec, x, w.t.get(), s);
@@ -1137,6 +1146,9 @@ void set_state_fine(Problem& p, double dt, double alpha, const double* U, const 
     vcast_d2f(f0.gexp[1].as<float>(), f0.gexp[0].as<double>(), f0.n_main_dofs, s);
   }
   for (int prec = 0; prec < 2; ++prec) op_precompute_frozen(f0.L, prec, s);
+  // a product's cell kernel starts early and reads the point values as constant data: keep a full
+  // completion between the pass that wrote them and the next product of the stream
+  if (f0.rows[0].get()) MFNS_CUDA(cudaMemsetAsync(f0.rows[0].get(), 0, 16, s));
 }
 
 void refresh_preconditioner(Problem& p, cudaStream_t s) {
@@ -1297,7 +1309,7 @@ BatchVcyclePtr make_batch_vcycle(const std::vector<Problem*>& ps, int prec, cons
       const Problem& p = *ps[i];
       if (t >= (int)p.levels.size() - 1) continue;
       const OpLaunch& L = p.levels[t]->L;
-      key[{L.dim, L.k, L.op, L.fq[prec] != nullptr, L.warps[prec], p.smoother, p.smoother_degree}].push_back(i);
+      key[{L.dim, L.k, L.op, L.fq[prec] || L.lq[prec], L.warps[prec], p.smoother, p.smoother_degree}].push_back(i);
     }
     for (auto& kv : key) {
       BatchGroup g;

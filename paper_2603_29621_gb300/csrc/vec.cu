@@ -1,5 +1,6 @@
 // Vector kernels (see vec.hpp).
 #include "common.hpp"
+#include "smoother.cuh"
 #include "vec.hpp"
 
 namespace mfns {
@@ -108,7 +109,7 @@ __global__ void k_distribute(T* x, const int32_t* dof, const int32_t* ptr, const
 template <typename T>
 __global__ void k_cheby(T* x, T* d, const T* b, const T* ax, const T* dinv, T c1, T c2, int64_t n) {
   GRID_STRIDE(i, n) {
-    const T di = (c1 != T(0) ? c1 * d[i] : T(0)) + c2 * dinv[i] * (b[i] - ax[i]);  // c1 = 0: d not read
+    const T di = smoother_direction(c1, c2, c1 != T(0) ? d[i] : T(0), dinv[i], b[i] - ax[i]);  // c1 = 0: d not read
     d[i] = di;
     x[i] += di;
   }
