@@ -131,8 +131,8 @@ __device__ __forceinline__ void mbar_wait0_bounded(unsigned addr, int* err) {
 // EPI: the fused smoother / residual epilogue is compiled in (structured launches only).
 // MULTI: one launch over the cells of several problems (structured, plain products); each block
 // reads its problem's fields from args.probs.
-// DEFER: one launch over every colour of a uniform level (blockIdx.y = colour) that writes each
-// cell's contributions to args.defer instead of adding them into dst (k_gather_cells sums them).
+// DEFER: one launch over every cell (structured: blockIdx.y = colour) that writes each cell's
+// contributions to args.defer instead of adding them into dst (k_gather_nodes sums them).
 template <int DIM, int K, int OP, typename T, bool STRUCT, bool DIAG, int FQ = 0, bool EPI = false,
           bool MULTI = false, bool DEFER = false>
 __global__ void __launch_bounds__(kOpWarps * 32, (EPI && OpMinBlocks<DIM, K, OP, T>::value > 1)
@@ -319,6 +319,28 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
 #pragma unroll
   for (int c = 0; c < NP; ++c) daccp[c] = 0;
 
+  if constexpr (Tr::FROZEN && FQ == 1) {
+    // the team's cell block (contiguous in global memory, a multiple of 16 bytes, 16-byte aligned)
+    // comes in with one TMA bulk copy issued by the team's first lane and tracked by the team's
+    // mbarrier; it overlaps the interpolation of the trial fields and is awaited before first use
+    constexpr unsigned BB = (unsigned)(FQB * sizeof(T));
+    static_assert(BB % 16 == 0, "bulk copies move multiples of 16 bytes");
+    if (lane_active && tid == 0) {
+      const unsigned sdst = (unsigned)__cvta_generic_to_shared(fqs);
+      const T* gsrc = fqd + (size_t)cellpos * FQB;
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mbar_addr) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar_addr), "r"(BB) : "memory");
+      asm volatile(
+          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(sdst),
+          "l"(gsrc), "r"(BB), "r"(mbar_addr)
+          : "memory");
+    }
+  }
+  // a deferred product starts while the previous kernel of the stream drains; that kernel may have
+  // written src (so src is not read as constant data here)
+  if constexpr (DEFER) asm volatile("griddepcontrol.wait;\n" ::: "memory");
   // vmult: issue the loads of src and of the dst values to be updated together with the
   // frozen state, so that each cell waits for global memory once
   T u0[NU][N];
@@ -329,11 +351,13 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
     for (int c = 0; c < N; ++c) {
       if constexpr (NU == 4) {
         if constexpr (sizeof(T) == 4) {
-          const float4 v = own ? __ldg(reinterpret_cast<const float4*>(srcp + node[c] * 4)) : make_float4(0, 0, 0, 0);
+          const float4* sp4 = reinterpret_cast<const float4*>(srcp + node[c] * 4);
+          const float4 v = own ? (DEFER ? *sp4 : __ldg(sp4)) : make_float4(0, 0, 0, 0);
           u0[0][c] = v.x; u0[1][c] = v.y; u0[2][c] = v.z; u0[3][c] = v.w;
         } else {
-          const double2 v0 = own ? __ldg(reinterpret_cast<const double2*>(srcp + node[c] * 4)) : make_double2(0, 0);
-          const double2 v1 = own ? __ldg(reinterpret_cast<const double2*>(srcp + node[c] * 4 + 2)) : make_double2(0, 0);
+          const double2* sp2 = reinterpret_cast<const double2*>(srcp + node[c] * 4);
+          const double2 v0 = own ? (DEFER ? sp2[0] : __ldg(sp2)) : make_double2(0, 0);
+          const double2 v1 = own ? (DEFER ? sp2[1] : __ldg(sp2 + 1)) : make_double2(0, 0);
           u0[0][c] = v0.x; u0[1][c] = v0.y; u0[2][c] = v1.x; u0[3][c] = v1.y;
         }
       } else {
@@ -378,25 +402,6 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
   T Ub[DIM][Q], Gb[DIM][DIM][Q], Rb[DIM][Q], tau[Q];
   T gp[DIM][Q], lb[DIM][Q], pb[Q];
   constexpr int NFQ = FrozenPoint<DIM>::NFQ;
-  if constexpr (Tr::FROZEN && FQ == 1) {
-    // the team's cell block (contiguous in global memory, a multiple of 16 bytes, 16-byte aligned)
-    // comes in with one TMA bulk copy issued by the team's first lane and tracked by the team's
-    // mbarrier; it overlaps the interpolation of the trial fields and is awaited before first use
-    constexpr unsigned BB = (unsigned)(FQB * sizeof(T));
-    static_assert(BB % 16 == 0, "bulk copies move multiples of 16 bytes");
-    if (lane_active && tid == 0) {
-      const unsigned sdst = (unsigned)__cvta_generic_to_shared(fqs);
-      const T* gsrc = fqd + (size_t)cellpos * FQB;
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mbar_addr) : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar_addr), "r"(BB) : "memory");
-      asm volatile(
-          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(sdst),
-          "l"(gsrc), "r"(BB), "r"(mbar_addr)
-          : "memory");
-    }
-  }
   if constexpr (Tr::FROZEN && FQ != 1) {
     T fz[DIM + 1][N];
 #pragma unroll
@@ -897,9 +902,12 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
           }
           if constexpr (DEFER) {
             const int slot = DIM == 3 ? (c * N + tj_n) * N + ti_n : c * N + ti_n;
-            T* pc = args.defer + ((size_t)cellpos * NB + slot) * NU;
-            if constexpr (NU == 4 && sizeof(T) == 4) {
-              *reinterpret_cast<float4*>(pc) = make_float4(r[0][c], r[1][c], r[2][c], r[3][c]);
+            T* pc = args.defer + ((size_t)cellpos * NB + slot) * defer_stride(NU);
+            if constexpr (NU >= 3 && sizeof(T) == 4) {
+              *reinterpret_cast<float4*>(pc) = make_float4(r[0][c], r[1][c], r[2][c], NU == 4 ? r[NU - 1][c] : T(0));
+            } else if constexpr (NU >= 3) {
+              *reinterpret_cast<double2*>(pc) = make_double2(r[0][c], r[1][c]);
+              *reinterpret_cast<double2*>(pc + 2) = make_double2(r[2][c], NU == 4 ? r[NU - 1][c] : T(0));
             } else {
 #pragma unroll
               for (int f = 0; f < NU; ++f) pc[f] = r[f][c];
@@ -928,7 +936,14 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
       }
       if (Tr::SPLIT_P && ownp) {
 #pragma unroll
-        for (int c = 0; c < NP; ++c) scatter_add(dstp + p_offset + pnode[c], rp[c]);
+        for (int c = 0; c < NP; ++c) {
+          if constexpr (DEFER) {
+            const int slot = DIM == 3 ? (c * NP + tj_p) * NP + ti_p : c * NP + ti_p;
+            args.defer_p[(size_t)cellpos * NBP + slot] = rp[c];
+          } else {
+            scatter_add(dstp + p_offset + pnode[c], rp[c]);
+          }
+        }
       }
     }
   }

@@ -109,12 +109,17 @@ struct OpArgs {
   const int32_t* block_pid;
   // device word in which a bounded wait that ran out sets bit 0 (or null)
   int* err;
-  // deferred product of a uniform level (one launch over every colour, blockIdx.y = colour): each
-  // cell's contributions go to defer[(cell position * nodes per cell + slot) * NU + f]; the cells of
-  // colour c start at cell position defer_off[c]
+  // deferred product (one launch over every cell; structured: blockIdx.y = colour, its cells from cell
+  // position defer_off[c] on): each cell's contributions go to defer[(cell position * nodes per cell
+  // + slot) * defer_stride(NU) + f], those of a Taylor--Hood pressure block to defer_p[cell position *
+  // pressure nodes per cell + slot]
   T* defer;
+  T* defer_p;
   int64_t defer_off[8];
 };
+
+// entries per node of a deferred contribution: three components are padded to one 16-byte word (FP32)
+__host__ __device__ constexpr int defer_stride(int nu) { return nu == 3 ? 4 : nu; }
 
 // ------------------------------------------------------------ small helpers
 template <typename T> struct V4;

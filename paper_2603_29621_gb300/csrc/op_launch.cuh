@@ -224,36 +224,75 @@ void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t 
   }
 }
 
-// Deferred product of a small uniform 3D level: one launch over every colour (blockIdx.y =
-// colour) writing each cell's contributions to `defer`; k_gather_cells forms dst from them.
+// Deferred product: one launch over every cell (structured: blockIdx.y = colour) writing the cells'
+// contributions to `defer` (and `defer_p`); k_gather_nodes forms the product from them.
 template <int DIM, int K, int OP, typename T>
-void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, cudaStream_t s) {
-  if constexpr (!(DIM == 3 && (OP == OP_STAB_NS || OP == OP_STOKES_A || OP == OP_PMASS))) {
-    throw Error(kErrUnsupported, "deferred products: 3D stabilised, vector-Laplacian or pressure-mass levels only");
-  } else {
-    constexpr int Q = K + 1, N = K + 1, NP = K + 1;
-    if (!L.structured || L.n_colors != 8) throw Error(kErrArg, "deferred products: uniform levels only");
-    OpArgs<T, Q, N, NP> a{};
-    fill_common(L, a);
-    a.src = src;
-    a.defer = defer;
-    using TM = Team<DIM, Q>;
-    const int prec = sizeof(T) == 8 ? 0 : 1;
-    const int warps = L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
-    const int cells_per_block = warps * TM::CPW;
-    int64_t off = 0, maxc = 0;
-    for (int c = 0; c < 8; ++c) {
+void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, T* defer_p, cudaStream_t s) {
+  constexpr int Q = K + 1, N = K + 1, NP = OP == OP_STOKES ? K : K + 1;
+  OpArgs<T, Q, N, NP> a{};
+  fill_common(L, a);
+  a.src = src;
+  a.defer = defer;
+  a.defer_p = defer_p;
+  using TM = Team<DIM, Q>;
+  const int prec = sizeof(T) == 8 ? 0 : 1;
+  const int warps = L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
+  const int cells_per_block = warps * TM::CPW;
+  int64_t maxc = L.n_cells;
+  unsigned gy = 1;
+  if (L.structured) {
+    gy = 1u << DIM;
+    int64_t off = 0;
+    maxc = 0;
+    for (unsigned c = 0; c < gy; ++c) {
       int64_t nc = 1;
       for (int d = 0; d < DIM; ++d) nc *= (L.n - ((c >> d) & 1) + 1) / 2;
       a.defer_off[c] = off;
       off += nc;
       maxc = std::max(maxc, nc);
     }
-    const dim3 grid((unsigned)((maxc + cells_per_block - 1) / cells_per_block), 8u);
-    op_kernel<DIM, K, OP, T, true, false, 0, false, false, true>
-        <<<grid, warps * 32, op_smem_bytes<DIM, K, OP, T>(warps, false), s>>>(a);
-    MFNS_CUDA(cudaGetLastError());
+  } else {
+    a.cell_begin = 0;
+    a.cell_end = (int32_t)L.n_cells;
   }
+  const dim3 grid((unsigned)((maxc + cells_per_block - 1) / cells_per_block), gy);
+  const bool timed = L.timer && L.timer->enabled;
+  if (timed) L.timer->record_pair_begin(s);
+  auto go = [&](auto kern, size_t sm) { launch_op(kern, grid, warps * 32, sm, s, a, true); };
+  bool staged = false;
+  if constexpr (OP == OP_STAB_NS) {
+    staged = a.fq != nullptr;  // point values staged per cell (2D and refined levels)
+    if (staged) {
+      const size_t sm = op_smem_bytes<DIM, K, OP, T>(warps, true);
+      static std::atomic<uint64_t> attr_done{0};  // per device, for the largest block size
+      int dev = 0;
+      MFNS_CUDA(cudaGetDevice(&dev));
+      const uint64_t bit = 1ull << (dev & 63);
+      if (!(attr_done.load() & bit)) {
+        const int mx = (int)op_smem_bytes<DIM, K, OP, T>(kOpWarps, true);
+        if constexpr (DIM == 2)
+          MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1, false, false, true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, false, false, 1, false, false, true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        attr_done.fetch_or(bit);
+      }
+      if (!L.structured)
+        go(op_kernel<DIM, K, OP, T, false, false, 1, false, false, true>, sm);
+      else if constexpr (DIM == 2)
+        go(op_kernel<DIM, K, OP, T, true, false, 1, false, false, true>, sm);
+      else
+        throw Error(kErrArg, "stored point values of a uniform 3D level: another layout");
+    }
+  }
+  if (!staged) {
+    const size_t sm = op_smem_bytes<DIM, K, OP, T>(warps, false);
+    if (L.structured)
+      go(op_kernel<DIM, K, OP, T, true, false, 0, false, false, true>, sm);
+    else
+      go(op_kernel<DIM, K, OP, T, false, false, 0, false, false, true>, sm);
+  }
+  if (timed) L.timer->record_pair_end(s);
 }
 
 template <int DIM, int K, int OP, typename T>
@@ -299,15 +338,14 @@ void op_launch_multi(const OpLaunch& L, int color, const MultiColour& mc, cudaSt
   }
 }
 
-#define MFNS_INSTANTIATE_DEFERRED(DIM, K, OP)                                                                  \
-  template void op_launch_deferred<DIM, K, OP, double>(const OpLaunch&, const double*, double*, cudaStream_t);    \
-  template void op_launch_deferred<DIM, K, OP, float>(const OpLaunch&, const float*, float*, cudaStream_t);
-
 #define MFNS_INSTANTIATE_OP(DIM, K, OP)                                                                        \
   template void op_launch<DIM, K, OP, double>(const OpLaunch&, const double*, double*, bool, cudaStream_t, int, int, \
                                                int64_t, const OpEpilogue*);                                        \
   template void op_launch<DIM, K, OP, float>(const OpLaunch&, const float*, float*, bool, cudaStream_t, int, int,    \
                                               int64_t, const OpEpilogue*);                                         \
+  template void op_launch_deferred<DIM, K, OP, double>(const OpLaunch&, const double*, double*, double*,           \
+                                                        cudaStream_t);                                             \
+  template void op_launch_deferred<DIM, K, OP, float>(const OpLaunch&, const float*, float*, float*, cudaStream_t); \
   template void op_launch_multi<DIM, K, OP, double>(const OpLaunch&, int, const MultiColour&, cudaStream_t);       \
   template void op_launch_multi<DIM, K, OP, float>(const OpLaunch&, int, const MultiColour&, cudaStream_t);
 

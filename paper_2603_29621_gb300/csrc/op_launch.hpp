@@ -105,15 +105,14 @@ struct MultiColour {
 template <int DIM, int K, int OP, typename T>
 void op_launch_multi(const OpLaunch& L, int color, const MultiColour& mc, cudaStream_t s);
 
-// Deferred product of a uniform 3D stabilised, vector-Laplacian or pressure-mass level (small
-// levels, where the eight colour launches are latency, not work): one launch over every colour writes each cell's
-// contributions to `defer` (n_cells * (k+1)^3 * NU entries of the precision), then one gather pass
-// forms dst = A src, every node summing its cells' contributions in colour order -- the additions
-// and the order of the colour-ordered scatter onto a cleared vector, so the result is the same bit
-// for bit -- with the identity rows (velocity of boundary nodes) src.
+// Deferred product: one launch over every cell writes the cells' contributions to `defer` (and those of a
+// Taylor--Hood pressure block to `defer_p`); gather_nodes (gather.hpp) adds, at every node, its cells'
+// contributions in colour order -- the additions and the order of the colour-ordered scatter onto a
+// cleared vector, so the product is the same bit for bit.
 template <int DIM, int K, int OP, typename T>
-void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, cudaStream_t s);
-void op_apply_deferred(const OpLaunch& L, int prec, const void* src, void* dst, void* defer, cudaStream_t s);
+void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, T* defer_p, cudaStream_t s);
+// p_at: offset of the pressure contributions in `defer`, in values
+void op_apply_deferred(const OpLaunch& L, int prec, const void* src, void* defer, int64_t p_at, cudaStream_t s);
 void op_apply_multi(const OpLaunch& L, int prec, int color, const MultiColour& mc, cudaStream_t s);
 
 // Runtime dispatch over (dim, k, op, precision); prec 0 = fp64, 1 = fp32.

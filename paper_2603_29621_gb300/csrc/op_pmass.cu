@@ -7,7 +7,4 @@ MFNS_INSTANTIATE_OP(2, 3, OP_PMASS)
 MFNS_INSTANTIATE_OP(3, 1, OP_PMASS)
 MFNS_INSTANTIATE_OP(3, 2, OP_PMASS)
 MFNS_INSTANTIATE_OP(3, 3, OP_PMASS)
-MFNS_INSTANTIATE_DEFERRED(3, 1, OP_PMASS)
-MFNS_INSTANTIATE_DEFERRED(3, 2, OP_PMASS)
-MFNS_INSTANTIATE_DEFERRED(3, 3, OP_PMASS)
 }  // namespace mfns

@@ -4,7 +4,4 @@ namespace mfns {
 MFNS_INSTANTIATE_OP(3, 1, OP_STAB_NS)
 MFNS_INSTANTIATE_OP(3, 2, OP_STAB_NS)
 MFNS_INSTANTIATE_OP(3, 3, OP_STAB_NS)
-MFNS_INSTANTIATE_DEFERRED(3, 1, OP_STAB_NS)
-MFNS_INSTANTIATE_DEFERRED(3, 2, OP_STAB_NS)
-MFNS_INSTANTIATE_DEFERRED(3, 3, OP_STAB_NS)
 }  // namespace mfns

@@ -5,8 +5,4 @@ MFNS_INSTANTIATE_OP(3, 1, OP_STOKES_A)
 MFNS_INSTANTIATE_OP(3, 2, OP_STOKES_A)
 MFNS_INSTANTIATE_OP(3, 3, OP_STOKES_A)
 MFNS_INSTANTIATE_OP(3, 4, OP_STOKES_A)
-MFNS_INSTANTIATE_DEFERRED(3, 1, OP_STOKES_A)
-MFNS_INSTANTIATE_DEFERRED(3, 2, OP_STOKES_A)
-MFNS_INSTANTIATE_DEFERRED(3, 3, OP_STOKES_A)
-MFNS_INSTANTIATE_DEFERRED(3, 4, OP_STOKES_A)
 }  // namespace mfns

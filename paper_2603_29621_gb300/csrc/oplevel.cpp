@@ -11,17 +11,22 @@
 
 namespace mfns {
 
-// uniform 3D stabilised / vector-Laplacian / pressure-mass levels of at most this many cells take
-// deferred products
+// Which products are deferred (one cell launch and a node pass) instead of one launch per colour: every
+// locally refined level (its 17 to 30 colours were most of a product: Stokes Q2/Q1, 24^3 cells with
+// two refinements, FP32 110 -> 70 us; the vector Laplacian's V-cycle on 16^3 with two refinements 1866 ->
+// 707 us), and uniform levels of at most this many cells (2D Stokes 16 x 16 FP64 19.6 -> 11.7 us; at
+// 24^3 Q3/Q2 FP64 the colours' launches are long enough to be the better ones, 341 against 352 us).
 #ifndef MFNS_DEFER_MAX_CELLS
 #define MFNS_DEFER_MAX_CELLS 4096
 #endif
 constexpr int64_t kDeferMaxCells = MFNS_DEFER_MAX_CELLS;
+constexpr int64_t kDeferMaxValues = int64_t(1) << 29;  // contributions of a level (4 GiB in FP64)
 
 size_t OpLevel::bytes() const {
   size_t b = fq[0].bytes() + fq[1].bytes() + cell_u.bytes() + cell_p.bytes() + cell_f.bytes() + mask.bytes() + constrained.bytes() +
              hang_dof.bytes() + hang_ptr.bytes() + hang_src.bytes() + pres.bytes() + tnodes.bytes() +
              tpnodes.bytes();
+  if (gather) b += gather->bytes();
   for (int i = 0; i < 2; ++i) b += rows[i].bytes() + hcell[i].bytes() + frozen[i].bytes() + hang_w[i].bytes() + dinv[i].bytes();
   return b;
 }
@@ -266,14 +271,11 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
     for (int32_t i : lv.constrained_host) km[(size_t)i >> 5] |= 1u << (i & 31);
     lv.keep_mask = upload(bud, km);
   }
-  // small uniform 3D stabilised (frozen state recomputed), vector-Laplacian and pressure-mass levels:
-  // products as one launch over all colours plus a gather pass (their eight colour launches are
-  // latency, not work)
-  if (lv.L.structured && !lv.L.lq[0] && (op == OP_STAB_NS || op == OP_STOKES_A || op == OP_PMASS) && dim == 3 &&
-      (int64_t)lv.L.n_cells <= kDeferMaxCells) {
-    const size_t entries = (size_t)lv.L.n_cells * (size_t)((k + 1) * (k + 1) * (k + 1)) * lv.NU;
-    for (int prec = 0; prec < 2; ++prec) lv.defer[prec].alloc(bud, entries * esize(prec));
-  }
+  if (op != OP_VMASS && !lv.L.lq[0])
+    for (int prec = 0; prec < 2; ++prec) {
+      lv.deferred[prec] = gather_fits(lv) && (!lv.L.structured || (int64_t)lv.L.n_cells <= kDeferMaxCells);
+      if (lv.deferred[prec]) ensure_gather(lv, prec, bud);
+    }
   lv.n_hang = (int64_t)hd.size();
   lv.hang_dof = upload(bud, hd);
   lv.hang_ptr = upload(bud, hp);
@@ -284,22 +286,83 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
   lv.pres = upload(bud, lv.pres_host);
 }
 
-void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cudaStream_t s) {
-  if (lv.hp) return hp_vmult(lv, prec, src, dst, s);
+// contributions of slot lists: node ids of every (cell position, slot), bit 31 ignored
+static void gather_table(const std::vector<int32_t>& nodes, int64_t n, std::vector<int32_t>& ptr,
+                         std::vector<int32_t>& idx) {
+  ptr.assign((size_t)n + 1, 0);
+  for (int32_t g : nodes) ++ptr[(size_t)(g & 0x7fffffff) + 1];
+  for (int64_t g = 0; g < n; ++g) ptr[g + 1] += ptr[g];
+  idx.resize(nodes.size());
+  std::vector<int32_t> at(ptr.begin(), ptr.end() - 1);
+  for (size_t e = 0; e < nodes.size(); ++e) idx[at[nodes[e] & 0x7fffffff]++] = (int32_t)e;
+}
+
+bool gather_fits(const OpLevel& lv) {
+  return !lv.hp && (int64_t)lv.L.n_cells * lv.nu.nb * (lv.NU == 3 ? 4 : lv.NU) <= kDeferMaxValues;
+}
+
+void ensure_gather(OpLevel& lv, int prec, Budget* bud) {
+  if (lv.hp) throw Error(kErrUnsupported, "deferred products of hp levels");
+  const size_t nc = lv.L.n_cells;
+  const bool th = lv.op == OP_STOKES;
+  if (!lv.gather) {
+    auto G = std::make_unique<NodeGather>();
+    G->nu = lv.NU;
+    G->n_main = lv.nu.n_nodes;
+    G->slots = (int64_t)nc * lv.nu.nb;
+    if (th) {
+      G->n_p = lv.np.n_nodes;
+      G->slots_p = (int64_t)nc * lv.np.nb;
+    }
+    std::vector<int32_t> ptr, idx;
+    auto slots = [&](const NodeSpace& sp) {  // masters in the colour order of the cell tables
+      std::vector<int32_t> v(nc * sp.nb);
+      for (size_t i = 0; i < nc; ++i)
+        for (int b = 0; b < sp.nb; ++b) v[i * sp.nb + b] = sp.cell_master[(size_t)lv.perm[i] * sp.nb + b];
+      return v;
+    };
+    gather_table(slots(lv.nu), G->n_main, ptr, idx);
+    G->ptr = upload(bud, ptr);
+    G->idx = upload(bud, idx);
+    if (th) {
+      gather_table(slots(lv.np), G->n_p, ptr, idx);
+      G->ptr_p = upload(bud, ptr);
+      G->idx_p = upload(bud, idx);
+    }
+    std::vector<uint8_t> mask((size_t)(G->n_main + G->n_p), 0);
+    for (int32_t i : lv.constrained_host) {
+      if (i < lv.n_main_dofs) mask[i / lv.NU] |= (uint8_t)(1u << (i % lv.NU));
+      else mask[G->n_main + (i - lv.n_main_dofs)] |= 1u;
+    }
+    G->mask = upload(bud, mask);
+    lv.gather = std::move(G);
+  }
+  NodeGather& G = *lv.gather;
+  if (!G.buf[prec].get()) G.buf[prec].alloc(bud, (size_t)(G.main_values() + G.slots_p) * esize(prec));
+}
+
+// a product whose node pass applies what follows it
+static void node_product(const OpLevel& lv, int prec, const NsAfterArgs& a, cudaStream_t s) {
   if (lv.L.lq[prec]) {
-    NsAfterArgs a;
-    a.dst = dst;
-    a.src = src;
-    ns_cells(lv.L, prec, src, lv.rows[prec].get(), s);
+    ns_cells(lv.L, prec, a.src, lv.rows[prec].get(), s);
     ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
     return;
   }
+  const NodeGather& G = *lv.gather;
+  op_apply_deferred(lv.L, prec, a.src, G.buf[prec].get(), G.main_values(), s);
+  gather_nodes(G, prec, a, s);
+}
+
+void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cudaStream_t s) {
+  if (lv.hp) return hp_vmult(lv, prec, src, dst, s);
+  if (oplevel_fuses(lv, prec)) {
+    NsAfterArgs a;
+    a.dst = dst;
+    a.src = src;
+    return node_product(lv, prec, a, s);
+  }
   // clearing kernel, then the colour launches (each may start before its predecessor drains);
   // on uniform meshes the clearing kernel also writes the identity rows, which no colour touches
-  if (lv.defer[prec].get()) {  // small uniform levels: one launch over all colours, one gather pass
-    op_apply_deferred(lv.L, prec, src, dst, lv.defer[prec].get(), s);
-    return;
-  }
   if (lv.keep_mask.get()) {
     op_apply_cleared(lv.L, prec, src, dst, lv.n_dofs, s, lv.keep_mask.as<uint32_t>());
     return;
@@ -312,7 +375,7 @@ void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cuda
     vcopy_idx<float>((float*)dst, (const float*)src, lv.constrained.as<int32_t>(), nc, s);
 }
 
-bool oplevel_fuses(const OpLevel& lv, int prec) { return lv.L.lq[prec] != nullptr; }
+bool oplevel_fuses(const OpLevel& lv, int prec) { return lv.L.lq[prec] || lv.deferred[prec]; }
 
 void oplevel_update(const OpLevel& lv, int prec, void* x, void* d, const void* b, const void* dinv, double c1,
                     double c2, cudaStream_t s) {
@@ -325,8 +388,7 @@ void oplevel_update(const OpLevel& lv, int prec, void* x, void* d, const void* b
   a.d = d;
   a.c1 = c1;
   a.c2 = c2;
-  ns_cells(lv.L, prec, x, lv.rows[prec].get(), s);
-  ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
+  node_product(lv, prec, a, s);
 }
 
 void oplevel_residual(const OpLevel& lv, int prec, const void* x, const void* b, void* r, cudaStream_t s) {
@@ -335,8 +397,7 @@ void oplevel_residual(const OpLevel& lv, int prec, const void* x, const void* b,
   a.dst = r;
   a.src = x;
   a.b = b;
-  ns_cells(lv.L, prec, x, lv.rows[prec].get(), s);
-  ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
+  node_product(lv, prec, a, s);
 }
 
 void oplevel_vmult_cols(const OpLevel& lv, int prec, const void* X, void* Y, int ncols, cudaStream_t s) {

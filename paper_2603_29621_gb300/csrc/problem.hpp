@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "common.hpp"
+#include "gather.hpp"
 #include "hp_space.hpp"
 #include "mesh.hpp"
 #include "opkind.hpp"
@@ -38,7 +39,8 @@ struct OpLevel {
   std::vector<int32_t> constrained_host;
   DevBuf constrained;                   // identity rows
   DevBuf keep_mask;                     // uniform meshes: bitmask of the identity rows (see oplevel_vmult)
-  DevBuf defer[2];                      // small uniform 3D levels: per-cell contributions (FP64 / FP32)
+  std::unique_ptr<NodeGather> gather;   // deferred products (and restrictions into this level)
+  bool deferred[2] = {false, false};    // products are deferred (FP64 / FP32)
   DevBuf rows[2];                       // uniform 3D stabilised levels: rows of a product (ns_lines.hpp)
   int64_t n_hang = 0;
   DevBuf hang_dof, hang_ptr, hang_src, hang_w[2];
@@ -110,6 +112,9 @@ void hp_asm_apply(const OpLevel& lv, int prec, const void* r, void* z, cudaStrea
 void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& ph, Budget* bud,
                    bool edge_dirichlet = false);
 void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cudaStream_t s);
+// the node table of a level without an hp structure, and its contribution buffer in one precision
+void ensure_gather(OpLevel& lv, int prec, Budget* bud);
+bool gather_fits(const OpLevel& lv);  // the contributions stay within a bound
 void oplevel_diag(const OpLevel& lv, int prec, void* diag, cudaStream_t s);
 // Levels whose product ends in a node pass that can apply what follows it (x, d, b in place of the
 // separate vector kernels): d = c1 d + c2 dinv (b - A x), x += d;  r = b - A x.

@@ -1148,7 +1148,8 @@ void set_state_fine(Problem& p, double dt, double alpha, const double* U, const 
   for (int prec = 0; prec < 2; ++prec) op_precompute_frozen(f0.L, prec, s);
   // a product's cell kernel starts early and reads the point values as constant data: keep a full
   // completion between the pass that wrote them and the next product of the stream
-  if (f0.rows[0].get()) MFNS_CUDA(cudaMemsetAsync(f0.rows[0].get(), 0, 16, s));
+  void* between = f0.rows[0].get() ? f0.rows[0].get() : f0.gather ? f0.gather->buf[0].get() : nullptr;
+  if (between) MFNS_CUDA(cudaMemsetAsync(between, 0, 16, s));
 }
 
 void refresh_preconditioner(Problem& p, cudaStream_t s) {

@@ -40,6 +40,7 @@ struct TransferArgs {
   const int32_t* fnodes;      // fine true node per slot: bit 31 skip, bit 30 boundary
   int32_t cell_begin, cell_end;
   int hkind;
+  T* defer;                   // restriction: contributions per (coarse cell, slot), or null: added into dst
 };
 
 // out = (Mz x My x Mx) in, matrices per direction selected by `sel` (0/1 half, 2 identity).
@@ -225,9 +226,15 @@ __global__ void __launch_bounds__(128) transfer_kernel(const TransferArgs<T, NF,
       for (int f = 0; f < NCOMP; ++f) apply_constraints<DIM, NC, true, T>(acc[f], buf, mask, tic, tjc, a.tab.Pc, ownc);
     if (valid && ownc) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c)
+      for (int c = 0; c < NC; ++c) {
+        const int slot = DIM == 3 ? (c * NC + tj) * NC + ti : c * NC + ti;
+        T* out = a.defer + (cell * NBC + slot) * defer_stride(NCOMP);
 #pragma unroll
-        for (int f = 0; f < NCOMP; ++f) scatter_add(a.dst + (int64_t)(cid[c] & 0x7fffffff) * NCOMP + f, acc[f][c]);
+        for (int f = 0; f < NCOMP; ++f) {
+          if (a.defer) out[f] = acc[f][c];
+          else scatter_add(a.dst + (int64_t)(cid[c] & 0x7fffffff) * NCOMP + f, acc[f][c]);
+        }
+      }
     }
   }
 }
@@ -319,6 +326,8 @@ void build_transfer(Transfer& t, const OpLevel& fine, const OpLevel& coarse, Bud
       }
     }
   const_cast<OpLevel&>(fine).tnodes = upload(bud, fn);
+  // restriction: contributions of every coarse cell in one launch, gathered per coarse node
+  for (int prec = 0; prec < 2 && gather_fits(coarse); ++prec) ensure_gather(const_cast<OpLevel&>(coarse), prec, bud);
   // 1D matrices
   std::vector<double> xf = gll_nodes(fine.k), xc = gll_nodes(coarse.k);
   t.E.assign(2 * NF * NC, 0.0);
@@ -358,6 +367,15 @@ static void launch_transfer(const Transfer& t, const OpLevel& fine, const OpLeve
     a.cell_end = (int32_t)t.n_coarse_cells;
     const unsigned grid = (unsigned)((t.n_coarse_cells + 4 * CPW - 1) / (4 * CPW));
     if (grid) transfer_kernel<DIM, NF, NC, NCOMP, NVEL, T, false><<<grid, 128, smem, s>>>(a);
+    MFNS_CUDA(cudaGetLastError());
+    return;
+  }
+  if (coarse.gather) {  // every coarse cell in one launch; transfer_restrict gathers
+    a.defer = coarse.gather->buf[sizeof(T) == 8 ? 0 : 1].template as<T>();
+    a.cell_begin = 0;
+    a.cell_end = (int32_t)t.n_coarse_cells;
+    const unsigned grid = (unsigned)((t.n_coarse_cells + 4 * CPW - 1) / (4 * CPW));
+    if (grid) transfer_kernel<DIM, NF, NC, NCOMP, NVEL, T, true><<<grid, 128, smem, s>>>(a);
     MFNS_CUDA(cudaGetLastError());
     return;
   }
@@ -650,11 +668,17 @@ void transfer_restrict(const Transfer& t, const OpLevel& fine, const OpLevel& co
   } else if (t.separable) {
     sep_restrict(t.sep, prec, rf, rc, s);
   } else {
-    MFNS_CUDA(cudaMemsetAsync(rc, 0, coarse.n_dofs * esize(prec), s));
+    if (!coarse.gather) MFNS_CUDA(cudaMemsetAsync(rc, 0, coarse.n_dofs * esize(prec), s));
     if (prec == 0)
       dispatch_transfer<double>(t, fine, coarse, (const double*)rf, (double*)rc, true, s);
     else
       dispatch_transfer<float>(t, fine, coarse, (const float*)rf, (float*)rc, true, s);
+    if (coarse.gather) {
+      NsAfterArgs a;  // sums per coarse node, constrained rows 0
+      a.after = 3;
+      a.dst = rc;
+      return gather_nodes(*coarse.gather, prec, a, s);
+    }
   }
   const int64_t nc = (int64_t)coarse.constrained_host.size();
   if (prec == 0)
