@@ -96,7 +96,8 @@ static NsProb<T> ns_prob(const OpLaunch& L, int prec, const T* src, void* rows) 
 // launch as a programmatic dependent of the previous kernel of the stream (both kernels here wait for
 // it before they touch what it writes)
 template <typename Kern, typename Args>
-static void launch_pdl(Kern kern, dim3 grid, unsigned block, size_t smem, cudaStream_t s, const Args& a) {
+static void launch_pdl(Kern kern, dim3 grid, unsigned block, size_t smem, cudaStream_t s, const Args& a,
+                       bool dependent = true) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
@@ -104,7 +105,7 @@ static void launch_pdl(Kern kern, dim3 grid, unsigned block, size_t smem, cudaSt
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   MFNS_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
@@ -122,6 +123,16 @@ static void set_smem(Kern kern, size_t bytes, std::atomic<uint64_t>& done) {
   done.fetch_or(bit);
 }
 
+// Shared memory of a cell launch, raised so that no SM takes more than its share of a grid that does not
+// fill the chip: a dependent launch finds some SMs free before others, and its blocks would pile up
+// there (V-cycles FP32 48^3 1115 -> 1086 us, 8^3 181 -> 173 us).
+static size_t spread_smem(size_t need, int64_t blocks) {
+  const int64_t per_sm = (blocks + 151) / 152;
+  if (per_sm > 16) return need;
+  const size_t share = (size_t)(228 * 1024 / per_sm - 1024) / 128 * 128;
+  return std::max(need, std::min(share, (size_t)227 * 1024));
+}
+
 bool ns_planes(int prec, int C) { return prec == 1 && C == 32; }
 
 template <int K, typename T, bool MULTI>
@@ -129,15 +140,19 @@ static void launch_cells(const NsArgs<T, K + 1>& a, int64_t blocks, int cmax, cu
   if constexpr (sizeof(T) == 4) {
     if (ns_planes(1, cmax)) {
       static std::atomic<uint64_t> done{0};
-      set_smem(k_ns_planes<K, MULTI>, NsPlane<K>::SMEM, done);
+      set_smem(k_ns_planes<K, MULTI>, 227 * 1024, done);
       return launch_pdl(k_ns_planes<K, MULTI>, dim3((unsigned)blocks), (unsigned)NsPlane<K>::THREADS,
-                        NsPlane<K>::SMEM, s, a);
+                        spread_smem(NsPlane<K>::SMEM, blocks), s, a);
     }
   }
+  // FP64 cells start on an idle chip, spread evenly over the SMs: every warp's operations take 64 cycles,
+  // and an early start that doubles the load of a few SMs costs more than the launch it hides (V-cycle
+  // 21^3 2417 -> 2367 us; 3170 us when the blocks may also pile up)
   using Sh = NsShape<K, T>;
   static std::atomic<uint64_t> done{0};
-  set_smem(k_ns_cells<K, T, MULTI>, Sh::smem(Sh::CMAX), done);
-  launch_pdl(k_ns_cells<K, T, MULTI>, dim3((unsigned)blocks), (unsigned)Sh::threads(cmax), Sh::smem(cmax), s, a);
+  set_smem(k_ns_cells<K, T, MULTI>, 227 * 1024, done);
+  launch_pdl(k_ns_cells<K, T, MULTI>, dim3((unsigned)blocks), (unsigned)Sh::threads(cmax),
+             spread_smem(Sh::smem(cmax), blocks), s, a, sizeof(T) == 4);
 }
 
 template <int K, typename T>
