@@ -135,13 +135,26 @@ void oplevel_distribute(const OpLevel& lv, int prec, void* x, cudaStream_t s);
 void oplevel_support(const OpLevel& lv, double* xyz, int* field);
 
 // Separable transfer between uniform meshes: 1D stencils P1 (fine x coarse) and P1^T per axis.
+struct SepDir {                         // one of them: rows = output nodes
+  DevBuf ptr, idx, w[2];
+  DevBuf lo, hi;                        // per row r: first / last input node of the rows >= r / <= r
+  int width = 1;                        // entries of the longest row
+  int rows[2] = {1, 1}, cols[2] = {1, 1};  // output tile of a block per precision
+  size_t smem[2] = {0, 0};
+};
 struct SepTransfer {
   int dim = 3, ncomp = 1, nvel = 0;
   int64_t Mf = 0, Mc = 0;               // 1D node counts
-  DevBuf p_ptr, p_idx, p_w[2];          // rows = fine nodes
-  DevBuf r_ptr, r_idx, r_w[2];          // rows = coarse nodes
+  SepDir p, r;                          // prolongation, restriction
   DevBuf i_ptr, i_idx, i_w;             // fine-to-coarse interpolation, rows = coarse nodes (fp64)
-  DevBuf tmp1[2], tmp2[2];              // intermediate grids per precision
+  DevBuf tmp1, tmp2;                    // intermediate grids of the state interpolation (fp64)
+};
+// First smoothing step of the coarse level, applied by the restriction that forms its right-hand side:
+// x = d = c2 dinv b.
+struct SepStart {
+  void *x = nullptr, *d = nullptr;
+  const void* dinv = nullptr;
+  double c2 = 0.0;
 };
 
 // Transfer between fine level (index l) and coarse level (l+1), Eq. 4.
@@ -173,7 +186,8 @@ struct HpTransfer {
 void build_transfer(Transfer& t, const OpLevel& fine, const OpLevel& coarse, Budget* bud,
                     bool allow_unrefined = false);
 bool build_separable(SepTransfer& t, const OpLevel& fine, const OpLevel& coarse, Budget* bud);
-void sep_restrict(const SepTransfer& t, int prec, const void* fine, void* coarse, cudaStream_t s);
+// (constrained coarse rows are set to zero)
+void sep_restrict(const SepTransfer& t, int prec, const void* fine, void* coarse, const SepStart* st, cudaStream_t s);
 // coarse = the fine FE function evaluated at the coarse nodes (all components, no masking; fp64)
 void sep_interpolate(const SepTransfer& t, const double* fine, double* coarse, cudaStream_t s);
 // the same for any transfer (separable passes, or per coarse cell through its children); the fine
@@ -183,8 +197,10 @@ void cell_interpolate(Transfer& t, const OpLevel& fine, const OpLevel& coarse, c
 void sep_prolongate_add(const SepTransfer& t, int prec, const void* coarse, void* fine, cudaStream_t s);
 void transfer_prolongate_add(const Transfer& t, const OpLevel& fine, const OpLevel& coarse, int prec,
                              const void* xc, void* xf, cudaStream_t s);
+// st: also start the coarse level's smoother; only where transfer_starts(t)
 void transfer_restrict(const Transfer& t, const OpLevel& fine, const OpLevel& coarse, int prec,
-                       const void* rf, void* rc, cudaStream_t s);
+                       const void* rf, void* rc, cudaStream_t s, const SepStart* st = nullptr);
+inline bool transfer_starts(const Transfer& t) { return !t.hp && t.separable; }
 
 struct Workspace {
   DevBuf r, d, t, b, x;                 // per level, per precision

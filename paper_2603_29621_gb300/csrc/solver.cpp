@@ -604,7 +604,7 @@ void setup_coarse(Problem& p, cudaStream_t s) {
 // ---------------------------------------------------------------------- smoothing
 template <typename T>
 static void smooth_op(const Problem& p, OpLevel& lv, Workspace& w, int prec, const T* b, T* x, bool x_is_zero,
-                      int degree, cudaStream_t s) {
+                      int degree, cudaStream_t s, bool started = false) {
   const int64_t n = lv.n_dofs;
   const T* dinv = lv.dinv[prec].as<T>();
   T* d = w.d.as<T>();
@@ -654,18 +654,19 @@ static void smooth_op(const Problem& p, OpLevel& lv, Workspace& w, int prec, con
   if (p.smoother == 1) {  // Jacobi relaxation
     const T omega = (T)(2.0 / (lmin + lmax));
     for (int it = 0; it < degree; ++it) {
-      if (it == 0 && x_is_zero)
-        vcheby0<T>(x, d, b, dinv, omega, n, s);
-      else
+      if (it == 0 && x_is_zero) {
+        if (!started) vcheby0<T>(x, d, b, dinv, omega, n, s);
+      } else {
         step(0.0, (double)omega);
+      }
     }
   } else {
     const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
     double rho_old = 1.0 / sigma;
-    if (x_is_zero)
-      vcheby0<T>(x, d, b, dinv, (T)(1.0 / theta), n, s);
-    else
+    if (!x_is_zero)
       step(0.0, 1.0 / theta);
+    else if (!started)
+      vcheby0<T>(x, d, b, dinv, (T)(1.0 / theta), n, s);
     for (int j = 1; j < degree; ++j) {
       const double rho = 1.0 / (2.0 * sigma - rho_old);
       step(rho * rho_old, 2.0 * rho / delta);
@@ -675,9 +676,16 @@ static void smooth_op(const Problem& p, OpLevel& lv, Workspace& w, int prec, con
   if (cur != x) vcopy<T>(x, cur, n, s);
 }
 
+// coefficient of the first step of a smoothing from zero, x = d = c dinv b
+static double smoother_start(const Problem& p, const OpLevel& lv) {
+  const double lmax = lv.lmax, lmin = lmax / 20.0;
+  return p.smoother == 1 ? 2.0 / (lmin + lmax) : 1.0 / (0.5 * (lmax + lmin));
+}
+
 template <typename T>
-static void smooth_t(Problem& p, int level, int prec, const T* b, T* x, bool x_is_zero, int degree, cudaStream_t s) {
-  smooth_op<T>(p, *p.levels[level], p.ws[prec][level], prec, b, x, x_is_zero, degree, s);
+static void smooth_t(Problem& p, int level, int prec, const T* b, T* x, bool x_is_zero, int degree, cudaStream_t s,
+                     bool started = false) {
+  smooth_op<T>(p, *p.levels[level], p.ws[prec][level], prec, b, x, x_is_zero, degree, s, started);
 }
 
 void smooth(Problem& p, int level, int prec, const void* b, void* x, bool x_is_zero, cudaStream_t s) {
@@ -698,7 +706,7 @@ static void coarse_solve(Problem& p, int prec, const T* b, T* x, cudaStream_t s)
 }
 
 template <typename T>
-static void vcycle_level(Problem& p, int prec, int l, const T* b, T* x, cudaStream_t s) {
+static void vcycle_level(Problem& p, int prec, int l, const T* b, T* x, cudaStream_t s, bool started = false) {
   const int L = (int)p.levels.size() - 1;
   if (l == L) {
     coarse_solve<T>(p, prec, b, x, s);
@@ -708,7 +716,7 @@ static void vcycle_level(Problem& p, int prec, int l, const T* b, T* x, cudaStre
   Workspace& w = p.ws[prec][l];
   Workspace& wc = p.ws[prec][l + 1];
   const int64_t n = lv.n_dofs;
-  smooth_t<T>(p, l, prec, b, x, true, p.smoother_degree, s);
+  smooth_t<T>(p, l, prec, b, x, true, p.smoother_degree, s, started);
   if (oplevel_fuses(lv, prec)) {
     oplevel_residual(lv, prec, x, b, w.r.get(), s);
   } else if (p.fused_smoother && lv.L.structured && lv.L.lastc) {
@@ -717,8 +725,15 @@ static void vcycle_level(Problem& p, int prec, int l, const T* b, T* x, cudaStre
     oplevel_vmult(lv, prec, x, w.t.get(), s);
     vsub<T>(w.r.as<T>(), b, w.t.as<T>(), n, s);
   }
-  transfer_restrict(*p.transfers[l], lv, *p.levels[l + 1], prec, w.r.get(), wc.b.get(), s);
-  vcycle_level<T>(p, prec, l + 1, wc.b.as<T>(), wc.x.as<T>(), s);
+  // the restriction also applies the first smoothing step of the next level (from zero)
+  const bool start = l + 1 < L && transfer_starts(*p.transfers[l]) && p.smoother_degree > 0;
+  SepStart st;
+  st.x = wc.x.get();
+  st.d = wc.d.get();
+  st.dinv = p.levels[l + 1]->dinv[prec].get();
+  st.c2 = smoother_start(p, *p.levels[l + 1]);
+  transfer_restrict(*p.transfers[l], lv, *p.levels[l + 1], prec, w.r.get(), wc.b.get(), s, start ? &st : nullptr);
+  vcycle_level<T>(p, prec, l + 1, wc.b.as<T>(), wc.x.as<T>(), s, start);
   transfer_prolongate_add(*p.transfers[l], lv, *p.levels[l + 1], prec, wc.x.get(), x, s);
   smooth_t<T>(p, l, prec, b, x, false, p.smoother_degree, s);
 }

@@ -656,7 +656,7 @@ void transfer_prolongate_add(const Transfer& t, const OpLevel& fine, const OpLev
 }
 
 void transfer_restrict(const Transfer& t, const OpLevel& fine, const OpLevel& coarse, int prec, const void* rf,
-                       void* rc, cudaStream_t s) {
+                       void* rc, cudaStream_t s, const SepStart* st) {
   if (t.hp) {
     MFNS_CUDA(cudaMemsetAsync(rc, 0, coarse.n_dofs * esize(prec), s));
     for (auto& g : t.hp->groups)
@@ -666,7 +666,7 @@ void transfer_restrict(const Transfer& t, const OpLevel& fine, const OpLevel& co
         dispatch_transfer<float>(g->t, g->fine_view, g->coarse_view, (const float*)rf, (float*)rc, true, s);
     if (coarse.hp) hp_condense(coarse, prec, rc, s);  // contributions of constrained entries to masters
   } else if (t.separable) {
-    sep_restrict(t.sep, prec, rf, rc, s);
+    return sep_restrict(t.sep, prec, rf, rc, st, s);
   } else {
     if (!coarse.gather) MFNS_CUDA(cudaMemsetAsync(rc, 0, coarse.n_dofs * esize(prec), s));
     if (prec == 0)
