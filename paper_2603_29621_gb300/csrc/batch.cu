@@ -19,7 +19,7 @@ struct MultiOp {
   std::vector<const void*> src;
   std::vector<void*> dst;
   std::vector<MultiColour> col;
-  NsMulti ns[2];   // uniform 3D stabilised levels: the members on the line and on the plane kernel
+  NsMulti ns[3];   // uniform 3D stabilised levels: the members on each cell kernel
   DevBuf probs, pid;
 };
 
@@ -34,28 +34,28 @@ static int64_t colour_cells(const OpLaunch& L, int c) {
 static void fill_ns(MultiOp& m, Budget* bud) {
   std::vector<char> desc;
   std::vector<int32_t> pid;
-  size_t desc_at[2], pid_at[2];
-  for (int planes = 0; planes < 2; ++planes) {
-    desc_at[planes] = desc.size();
-    pid_at[planes] = pid.size();
+  size_t desc_at[3], pid_at[3];
+  for (int kind = 0; kind < 3; ++kind) {
+    desc_at[kind] = desc.size();
+    pid_at[kind] = pid.size();
     int members = 0;
     for (size_t i = 0; i < m.lv.size(); ++i) {
       const OpLevel& lv = *m.lv[i];
-      if (ns_planes(m.prec, lv.L.lc[m.prec]) != (planes == 1)) continue;
+      if (ns_kernel(lv.L, m.prec) != kind) continue;
       const int64_t nb = ns_blocks(lv.L, m.prec);
       if (pid.size() + (size_t)nb >= (size_t)1 << 31)
         throw Error(kErrUnsupported, "multi-problem launch: too many blocks");
-      ns_descriptor(lv.L, m.prec, m.src[i], lv.rows[m.prec].get(), (int32_t)(pid.size() - pid_at[planes]), desc);
+      ns_descriptor(lv.L, m.prec, m.src[i], lv.rows[m.prec].get(), (int32_t)(pid.size() - pid_at[kind]), desc);
       pid.insert(pid.end(), (size_t)nb, members++);
-      m.ns[planes].cmax = std::max(m.ns[planes].cmax, lv.L.lc[m.prec]);
+      m.ns[kind].cmax = std::max(m.ns[kind].cmax, lv.L.lc[m.prec]);
     }
-    m.ns[planes].blocks = (int64_t)(pid.size() - pid_at[planes]);
+    m.ns[kind].blocks = (int64_t)(pid.size() - pid_at[kind]);
   }
   m.probs = upload(bud, desc);
   m.pid = upload(bud, pid);
-  for (int planes = 0; planes < 2; ++planes) {
-    m.ns[planes].probs = m.probs.as<char>() + desc_at[planes];
-    m.ns[planes].block_pid = m.pid.as<int32_t>() + pid_at[planes];
+  for (int kind = 0; kind < 3; ++kind) {
+    m.ns[kind].probs = m.probs.as<char>() + desc_at[kind];
+    m.ns[kind].block_pid = m.pid.as<int32_t>() + pid_at[kind];
   }
 }
 
@@ -138,7 +138,7 @@ MultiOp* multi_op_create(const std::vector<const OpLevel*>& lv, const std::vecto
 
 // dst_i = A_i src_i for every member (constrained rows dst = src), one launch per colour.
 void multi_vmult(const MultiOp& m, cudaStream_t s) {
-  if (m.ns[0].blocks || m.ns[1].blocks) {
+  if (m.ns[0].blocks || m.ns[1].blocks || m.ns[2].blocks) {
     for (const NsMulti& part : m.ns)
       if (part.blocks) ns_cells_multi(*m.L0, m.prec, part, s);
     for (size_t i = 0; i < m.lv.size(); ++i) {

@@ -13,18 +13,29 @@ bool ns_lines(const OpLaunch& L) {
   return L.op == OP_STAB_NS && L.dim == 3 && L.structured && L.k >= 1 && L.k <= 3;
 }
 
-// Cells per block.  FP32: 32 (full warps), fewer while the level has less than one block per SM.
-// FP64: four warps per block where the chip gets many, else two (finer balance), and one
-// (k = 2: 27 of 32 lanes) on levels that do not fill the SMs' four FP64 issue ports.
+// Which cell kernel, and the cells per block.  FP32: planes with 32 cells (full warps) where that gives
+// every SM a block, else lines with fewer cells.  FP64: lines with four warps per block where the
+// chip gets many, else two (finer balance); items on levels that do not fill the SMs' FP64 issue
+// ports, with cells for one item per thread and stage, or a third of them on the smallest.
 int ns_cells_per_block(int k, int prec, int64_t cells) {
+  const int nl = (k + 1) * (k + 1);
   if (prec == 1) {
     int C = 32;
     while (C > 4 && cells / C < 152) C /= 2;
     return C;
   }
-  const int four = 128 / ((k + 1) * (k + 1)), two = 64 / ((k + 1) * (k + 1)), one = 32 / ((k + 1) * (k + 1));
-  return cells / four >= 152 * 8 ? four : cells / two >= 152 * 2 ? two : one;
+  const int items = 32 / nl, least = k == 1 ? 2 : 1;
+  if (cells <= 152 * 4 * least) return least;
+  if (cells <= 152 * 4 * items) return items;
+  return cells / (128 / nl) >= 152 * 8 ? 128 / nl : 64 / nl;
 }
+
+enum NsKernel { kLines, kPlanes, kItems };
+static NsKernel kernel_of(int k, int prec, int C) {
+  if (prec == 1) return C == 32 ? kPlanes : kLines;
+  return C <= 32 / ((k + 1) * (k + 1)) ? kItems : kLines;
+}
+int ns_kernel(const OpLaunch& L, int prec) { return kernel_of(L.k, prec, L.lc[prec]); }
 
 int64_t ns_blocks(const OpLaunch& L, int prec) {
   const int64_t cells = (int64_t)L.n * L.n * L.n;
@@ -70,6 +81,17 @@ static void fill_tab(const OpLaunch& L, NsTab<T, Q>& t) {
       t.D2S[i][a] = (T)(-lapc * d2s);
       t.Dw[i][a] = (T)(L.D[a * Q + i] * L.W[a] / L.W[i]);
     }
+  auto halves = [](const T (&m)[Q][Q], T (&h)[2]) {
+    h[0] = (T)(0.5 * ((double)m[0][0] + (double)m[0][Q - 1]));
+    h[1] = (T)(0.5 * ((double)m[0][0] - (double)m[0][Q - 1]));
+  };
+  halves(t.S, t.hS);
+  halves(t.Sp, t.hSp);
+  halves(t.D, t.hD);
+  halves(t.St, t.hSt);
+  halves(t.Dw, t.hDw);
+  halves(t.Sf, t.hSf);
+  halves(t.Sfp, t.hSfp);
 }
 
 template <typename T>
@@ -133,26 +155,34 @@ static size_t spread_smem(size_t need, int64_t blocks) {
   return std::max(need, std::min(share, (size_t)227 * 1024));
 }
 
-bool ns_planes(int prec, int C) { return prec == 1 && C == 32; }
-
 template <int K, typename T, bool MULTI>
 static void launch_cells(const NsArgs<T, K + 1>& a, int64_t blocks, int cmax, cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) {
-    if (ns_planes(1, cmax)) {
-      static std::atomic<uint64_t> done{0};
-      set_smem(k_ns_planes<K, MULTI>, 227 * 1024, done);
-      return launch_pdl(k_ns_planes<K, MULTI>, dim3((unsigned)blocks), (unsigned)NsPlane<K>::THREADS,
-                        spread_smem(NsPlane<K>::SMEM, blocks), s, a);
-    }
-  }
+  const NsKernel kind = kernel_of(K, sizeof(T) == 4, cmax);
+  const dim3 grid((unsigned)blocks);
   // FP64 cells start on an idle chip, spread evenly over the SMs: every warp's operations take 64 cycles,
   // and an early start that doubles the load of a few SMs costs more than the launch it hides (V-cycle
   // 21^3 2417 -> 2367 us; 3170 us when the blocks may also pile up)
+  const bool early = sizeof(T) == 4;
+  if constexpr (sizeof(T) == 8) {
+    if (kind == kItems) {
+      static std::atomic<uint64_t> done{0};
+      set_smem(k_ns_items<K, MULTI>, 227 * 1024, done);
+      return launch_pdl(k_ns_items<K, MULTI>, grid, NsItems<K>::THREADS, spread_smem(NsItems<K>::smem(cmax), blocks), s,
+                        a, early);
+    }
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (kind == kPlanes) {
+      static std::atomic<uint64_t> done{0};
+      set_smem(k_ns_planes<K, MULTI>, 227 * 1024, done);
+      return launch_pdl(k_ns_planes<K, MULTI>, grid, NsPlane<K>::THREADS, spread_smem(NsPlane<K>::SMEM, blocks), s, a);
+    }
+  }
   using Sh = NsShape<K, T>;
   static std::atomic<uint64_t> done{0};
   set_smem(k_ns_cells<K, T, MULTI>, 227 * 1024, done);
-  launch_pdl(k_ns_cells<K, T, MULTI>, dim3((unsigned)blocks), (unsigned)Sh::threads(cmax),
-             spread_smem(Sh::smem(cmax), blocks), s, a, sizeof(T) == 4);
+  launch_pdl(k_ns_cells<K, T, MULTI>, grid, (unsigned)Sh::threads(cmax), spread_smem(Sh::smem(cmax), blocks), s, a,
+             early);
 }
 
 template <int K, typename T>

@@ -23,7 +23,7 @@
 // and for several in a launch.
 //
 // Measured against eight colour launches of the warp-per-three-cells kernel (whole product, GB300): Q2
-// 64^3 FP32 176 -> 130 us, 48^3 FP64 1849 -> 1158 us (FP64 pipe 87 % busy), Q3 31^3 FP32 61.8 -> 60.1 us,
+// 64^3 FP32 176 -> 129 us, 48^3 FP64 1849 -> 1114 us (FP64 pipe 87 % busy), Q3 31^3 FP32 61.8 -> 60.1 us,
 // five Q1 45^3 FP32 smoothing sweeps 116 -> 52 us.  The FP32 cell launch (103 us at 64^3) is bound by
 // the DRAM stream of the point values (5.4 TB/s), the node pass (28 us) by its rows.
 #pragma once
@@ -47,6 +47,8 @@ struct NsTab {
   T DS[Q][Q];   // derivative at the Gauss points from nodal values
   T D2S[Q][Q];  // second derivative from nodal values, scaled as D2
   T Sfp[Q][Q];  // last test stage of the pressure (h^2 times the sign of the continuity row)
+  // Q = 3: half the sum and half the difference of the first row's outer entries, of S, Sp, D, St, Dw, Sf, Sfp
+  T hS[2], hSp[2], hD[2], hSt[2], hDw[2], hSf[2], hSfp[2];
 };
 
 template <typename T>
@@ -111,10 +113,10 @@ enum NsRow { kDense, kTrial, kTest };
 // symmetric table; for Q = 3: kTrial: the centre row is a multiple of (0, 1, 0); kTest: the centre
 // column is, and unless SCALED its entry is 1
 template <int Q, NsRow R, bool SCALED, typename T>
-__device__ __forceinline__ void line_sym(const T (&M)[Q][Q], const T (&u)[Q], T (&o)[Q]) {
+__device__ __forceinline__ void line_sym(const T (&M)[Q][Q], const T (&h)[2], const T (&u)[Q], T (&o)[Q]) {
   if constexpr (Q == 3 && R != kDense) {
     const T e = u[0] + u[2], d = u[0] - u[2];
-    const T pe = T(0.5) * (M[0][0] + M[0][2]), po = T(0.5) * (M[0][0] - M[0][2]);
+    const T pe = h[0], po = h[1];
     if constexpr (R == kTrial) {
       const T E = fma(pe, e, M[0][1] * u[1]);
       o[0] = fma(po, d, E);
@@ -138,13 +140,13 @@ __device__ __forceinline__ void line_sym(const T (&M)[Q][Q], const T (&u)[Q], T 
 }
 // derivative at the Gauss points and, with SECOND, the scaled second derivative (Q = 3: one value)
 template <int Q, bool SECOND, typename T>
-__device__ __forceinline__ void line_deriv(const T (&D)[Q][Q], const T (&D2)[Q][Q], const T (&u)[Q], T (&o)[Q],
-                                           T (&x)[Q]) {
+__device__ __forceinline__ void line_deriv(const T (&D)[Q][Q], const T (&h)[2], const T (&D2)[Q][Q], const T (&u)[Q],
+                                           T (&o)[Q], T (&x)[Q]) {
   if constexpr (Q == 3) {
     // rows (a, b, c), (-d, 0, d), (-c, -b, -a) with a + b + c = 0; D2 rows q (1, -2, 1)
     const T e = u[0] + u[2], d = u[0] - u[2];
     const T t = fma(T(-0.5), e, u[1]);
-    const T m = T(0.5) * (D[0][0] - D[0][2]) * d;
+    const T m = mul_rn(h[1], d);
     o[0] = fma(D[0][1], t, m);
     o[2] = fma(-D[0][1], t, m);
     o[1] = mul_rn(D[1][0], d);
@@ -168,10 +170,10 @@ __device__ __forceinline__ void line_deriv(const T (&D)[Q][Q], const T (&D2)[Q][
 }
 // o = Dw u, or with ADD o += Dw u
 template <int Q, bool ADD, typename T>
-__device__ __forceinline__ void line_dwt(const T (&Dw)[Q][Q], const T (&u)[Q], T (&o)[Q]) {
+__device__ __forceinline__ void line_dwt(const T (&Dw)[Q][Q], const T (&h)[2], const T (&u)[Q], T (&o)[Q]) {
   if constexpr (Q == 3) {
     const T e = u[0] + u[2], d = u[0] - u[2];
-    const T m = T(0.5) * (Dw[0][0] + Dw[0][2]), k = T(0.5) * (Dw[0][0] - Dw[0][2]);
+    const T m = h[0], k = h[1];
     const T X = fma(m, e, Dw[0][1] * u[1]);
     o[0] = fma(k, d, ADD ? o[0] + X : X);
     o[2] = fma(k, d, ADD ? o[2] - X : -X);
@@ -239,7 +241,9 @@ struct NsShape {
   static constexpr bool STAGE = sizeof(T) == 4 && Q < 4;
   static constexpr int CMAX = UNI ? 32 : 128 / NL;
   static constexpr int THREADS = UNI ? NL * 32 : 128;
-  static constexpr int MINB = UNI ? (Q == 2 ? 6 : Q == 3 ? 2 : 1) : (Q == 4 ? 3 : 4);
+  // FP64: five blocks' worth of registers (spilling a little); with four, the 1,323 blocks of a 21^3 level
+  // need a second round (V-cycle 1863 -> 1795 us)
+  static constexpr int MINB = UNI ? (Q == 2 ? 6 : Q == 3 ? 2 : 1) : (Q == 4 ? 3 : 5);
   static constexpr int NXX = !LINES || Q == 2 ? 0 : Q == 3 ? NL : NL * Q;  // second-derivative entries per cell
   __host__ __device__ static constexpr int slots(int C) { return UNI ? 32 : C; }
   __host__ __device__ static constexpr size_t buf_values(int C) { return (size_t)NL * Q * 4 * slots(C); }
@@ -360,8 +364,8 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     }
     T o[4][Q];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) line_sym<Q, kTrial, false>(tab.S, u[f], o[f]);
-    line_sym<Q, kTrial, true>(tab.Sp, u[3], o[3]);
+    for (int f = 0; f < 3; ++f) line_sym<Q, kTrial, false>(tab.S, tab.hS, u[f], o[f]);
+    line_sym<Q, kTrial, true>(tab.Sp, tab.hSp, u[3], o[3]);
     if (work)
 #pragma unroll
       for (int a = 0; a < Q; ++a) ns_st(A, px + a, slot, ls, o[0][a], o[1][a], o[2][a], o[3][a]);
@@ -385,7 +389,7 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     T u[4][Q], o[4][Q];
     load_line(A, py, Q, u);
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_sym<Q, kTrial, false>(tab.S, u[f], o[f]);
+    for (int f = 0; f < 4; ++f) line_sym<Q, kTrial, false>(tab.S, tab.hS, u[f], o[f]);
     store_line(A, py, Q, o);  // a thread's own entries: in place
   }
   __syncthreads();
@@ -394,12 +398,12 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     T u[4][Q];
     load_line(A, pz, Q * Q, u);
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_sym<Q, kTrial, false>(tab.S, u[f], val[f]);
+    for (int f = 0; f < 4; ++f) line_sym<Q, kTrial, false>(tab.S, tab.hS, u[f], val[f]);
     store_line(A, pz, Q * Q, val);
     T dummy[Q];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.D2, val[f], dz[f], lz[f]);
-    line_deriv<Q, false>(tab.D, tab.D2, val[3], dz[3], dummy);
+    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.hD, tab.D2, val[f], dz[f], lz[f]);
+    line_deriv<Q, false>(tab.D, tab.hD, tab.D2, val[3], dz[3], dummy);
   }
   __syncthreads();
   if constexpr (Sh::LINES) {
@@ -408,8 +412,8 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     T u[4][Q], o[4][Q], x2[3][Q], dummy[Q];
     load_line(A, px, 1, u);
 #pragma unroll
-    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.D2, u[f], o[f], x2[f]);
-    line_deriv<Q, false>(tab.D, tab.D2, u[3], o[3], dummy);
+    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.hD, tab.D2, u[f], o[f], x2[f]);
+    line_deriv<Q, false>(tab.D, tab.hD, tab.D2, u[3], o[3], dummy);
 #pragma unroll
     for (int a = 0; a < Q; ++a)
       if (Q > 2) o[3][a] += x2[0][a];
@@ -423,8 +427,8 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     }
     load_line(A, py, Q, u);
 #pragma unroll
-    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.D2, u[f], o[f], x2[f]);
-    line_deriv<Q, false>(tab.D, tab.D2, u[3], o[3], dummy);
+    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.hD, tab.D2, u[f], o[f], x2[f]);
+    line_deriv<Q, false>(tab.D, tab.hD, tab.D2, u[3], o[3], dummy);
 #pragma unroll
     for (int a = 0; a < Q; ++a)
       if (Q > 2) o[3][a] += x2[1][a];
@@ -522,18 +526,18 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     }
   }
 #pragma unroll
-  for (int f = 0; f < 4; ++f) line_dwt<Q, true>(tab.Dw, cz4[f], acc[f]);
+  for (int f = 0; f < 4; ++f) line_dwt<Q, true>(tab.Dw, tab.hDw, cz4[f], acc[f]);
   __syncthreads();
   // ---- test side: transposed derivatives, then the transposed values z, y, x
   if constexpr (Sh::LINES) {
     T u[4][Q], o[4][Q];
     load_line(B, px, 1, u);
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_dwt<Q, false>(tab.Dw, u[f], o[f]);
+    for (int f = 0; f < 4; ++f) line_dwt<Q, false>(tab.Dw, tab.hDw, u[f], o[f]);
     store_line(B, px, 1, o);
     load_line(G, py, Q, u);
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_dwt<Q, false>(tab.Dw, u[f], o[f]);
+    for (int f = 0; f < 4; ++f) line_dwt<Q, false>(tab.Dw, tab.hDw, u[f], o[f]);
     store_line(G, py, Q, o);
     __syncthreads();
 #pragma unroll
@@ -560,7 +564,7 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
   {
     T o[4][Q];
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_sym<Q, kTest, false>(tab.St, acc[f], o[f]);
+    for (int f = 0; f < 4; ++f) line_sym<Q, kTest, false>(tab.St, tab.hSt, acc[f], o[f]);
     store_line(A, pz, Q * Q, o);
   }
   __syncthreads();
@@ -568,7 +572,7 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     T u[4][Q], o[4][Q];
     load_line(A, py, Q, u);
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_sym<Q, kTest, false>(tab.St, u[f], o[f]);
+    for (int f = 0; f < 4; ++f) line_sym<Q, kTest, false>(tab.St, tab.hSt, u[f], o[f]);
     store_line(A, py, Q, o);
   }
   __syncthreads();
@@ -577,8 +581,8 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     T u[4][Q];
     load_line(A, px, 1, u);
 #pragma unroll
-    for (int f = 0; f < 3; ++f) line_sym<Q, kTest, true>(tab.Sf, u[f], r[f]);
-    line_sym<Q, kTest, true>(tab.Sfp, u[3], r[3]);
+    for (int f = 0; f < 3; ++f) line_sym<Q, kTest, true>(tab.Sf, tab.hSf, u[f], r[f]);
+    line_sym<Q, kTest, true>(tab.Sfp, tab.hSfp, u[3], r[3]);
   }
   // ---- the face between x-neighbours of the block, then the node values of the row
   T left[4];
@@ -609,6 +613,187 @@ k_ns_cells(const __grid_constant__ NsArgs<T, K + 1> args) {
     if (cx == n - 1) put(out + 4 * K, r[0][K], r[1][K], r[2][K], r[3][K]);
     else if (lane == C - 1)
       put(P.tails + ((int64_t)blk * NL + w) * 4, r[0][K], r[1][K], r[2][K], r[3][K]);
+  }
+}
+
+// ------------------------------------------------------------------------------------ small FP64 levels: items
+// FP64 levels that do not fill the chip: a block of 128 threads works on C cells, and every stage splits its
+// work into items of one field of one line, or one point, over all threads; the fields live in shared
+// memory between the stages.  A thread then does a quarter of the operations that a line's owner does,
+// which is the time of a small FP64 level: one warp's FP64 operations take 64 cycles each.  Warps are
+// rotated by the block index, because a stage with few items would otherwise always load the same
+// quarter of the SM.
+template <int K>
+struct NsItems {
+  static constexpr int Q = K + 1, NL = Q * Q, NP = NL * Q, THREADS = 128;
+  static constexpr int NX = Q == 2 ? 0 : Q == 3 ? NL : NP;  // second derivatives per direction and field
+  static constexpr int CELL = 16 * NP + 9 * NX;              // values of a cell
+  __host__ __device__ static constexpr size_t smem(int C) { return (size_t)CELL * C * 8; }
+};
+
+template <int K, bool MULTI>
+__global__ void __launch_bounds__(128) k_ns_items(const __grid_constant__ NsArgs<double, K + 1> args) {
+  using T = double;
+  using It = NsItems<K>;
+  constexpr int Q = K + 1, NL = Q * Q, NP = NL * Q, NX = It::NX;
+  extern __shared__ __align__(128) unsigned char ns_smem[];
+  const NsDesc<T, Q>& desc = MULTI ? args.probs[args.block_pid[blockIdx.x]] : args.one;
+  const NsTab<T, Q>& tab = desc.tab;
+  const NsProb<T>& P = desc.p;
+  const int blk = (int)blockIdx.x - (MULTI ? P.first_block : 0);
+  const int C = P.C, n = P.n, M = K * n + 1;
+  const int tid = (int)((threadIdx.x + 32u * (blockIdx.x & 3u)) & 127u);
+  T* mem = reinterpret_cast<T*>(ns_smem);
+  // per cell: U[4][NP] (values, then sums), G[3][4][NP] (derivatives, then their coefficients), X[3][3][NX]
+  auto U = [&](int c, int f) { return mem + c * It::CELL + f * NP; };
+  auto G = [&](int c, int d, int f) { return mem + c * It::CELL + (4 + 4 * d + f) * NP; };
+  auto X = [&](int c, int d, int f) { return mem + c * It::CELL + 16 * NP + (3 * d + f) * NX; };
+  const uint32_t t0 = (uint32_t)blk * (uint32_t)C;
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  auto line = [](int dir, int w, int& p0, int& st) {  // entries of line w along dir
+    p0 = dir == 0 ? Q * w : dir == 1 ? w % Q + Q * Q * (w / Q) : w;
+    st = dir == 0 ? 1 : dir == 1 ? Q : Q * Q;
+  };
+  // ---- trial values: x (from the nodal values), y, z
+  for (int it = tid; it < C * 4 * NL; it += 128) {
+    const int c = it / (4 * NL), f = it / NL % 4, w = it % NL;
+    const uint32_t t = min(t0 + (uint32_t)c, P.cells - 1);
+    const int cx = (int)(t % (uint32_t)n), row = (int)(t / (uint32_t)n), cy = row % n, cz = row / n;
+    const int iy = K * cy + w % Q, iz = K * cz + w / Q;
+    const bool bl = iy == 0 || iy == M - 1 || iz == 0 || iz == M - 1;
+    const T* s = P.src + ((int64_t)(K * cx) + (int64_t)M * ((int64_t)iy + (int64_t)M * iz)) * 4 + f;
+    T u[Q], o[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      u[a] = s[4 * a];
+      if (f < 3 && (bl || (a == 0 && cx == 0) || (a == K && cx == n - 1))) u[a] = T(0);
+    }
+    if (f < 3) line_sym<Q, kTrial, false>(tab.S, tab.hS, u, o);
+    else line_sym<Q, kTrial, true>(tab.Sp, tab.hSp, u, o);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) U(c, f)[Q * w + a] = o[a];
+  }
+#pragma unroll
+  for (int dir = 1; dir < 3; ++dir) {
+    __syncthreads();
+    for (int it = tid; it < C * 4 * NL; it += 128) {
+      const int c = it / (4 * NL), f = it / NL % 4, w = it % NL;
+      int p0, st;
+      line(dir, w, p0, st);
+      T u[Q], o[Q];
+#pragma unroll
+      for (int a = 0; a < Q; ++a) u[a] = U(c, f)[p0 + st * a];
+      line_sym<Q, kTrial, false>(tab.S, tab.hS, u, o);
+#pragma unroll
+      for (int a = 0; a < Q; ++a) U(c, f)[p0 + st * a] = o[a];
+    }
+  }
+  __syncthreads();
+  // ---- derivatives along every line
+  for (int it = tid; it < C * 12 * NL; it += 128) {
+    const int c = it / (12 * NL), d = it / (4 * NL) % 3, f = it / NL % 4, w = it % NL;
+    int p0, st;
+    line(d, w, p0, st);
+    T u[Q], o[Q], x2[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) u[a] = U(c, f)[p0 + st * a];
+    line_deriv<Q, true>(tab.D, tab.hD, tab.D2, u, o, x2);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) G(c, d, f)[p0 + st * a] = o[a];
+    if (f < 3) {
+      if (Q == 3) X(c, d, f)[w] = x2[0];
+      else if (Q > 3)
+#pragma unroll
+        for (int a = 0; a < Q; ++a) X(c, d, f)[p0 + st * a] = x2[a];
+    }
+  }
+  __syncthreads();
+  // ---- pointwise terms
+  for (int it = tid; it < C * NP; it += 128) {
+    const int c = it / NP, p = it % NP, i = p % Q, j = p / Q % Q, l = p / NL;
+    T F[4][4], v[4], gx[4], gy[4], gz[4], lap[3], c0[4], cxp[4], cyp[4], czp[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double2 a = __ldg(reinterpret_cast<const double2*>(P.fq + ns_fq_at<T, Q>(blk, p % NL, l, q, 0, c, C)));
+      const double2 b = __ldg(reinterpret_cast<const double2*>(P.fq + ns_fq_at<T, Q>(blk, p % NL, l, q, 1, c, C)));
+      F[q][0] = a.x; F[q][1] = a.y; F[q][2] = b.x; F[q][3] = b.y;
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      v[f] = U(c, f)[p];
+      gx[f] = G(c, 0, f)[p];
+      gy[f] = G(c, 1, f)[p];
+      gz[f] = G(c, 2, f)[p];
+    }
+#pragma unroll
+    for (int f = 0; f < 3; ++f)
+      lap[f] = Q == 2 ? T(0)
+                      : (X(c, 0, f)[Q == 3 ? j + Q * l : p] + X(c, 1, f)[Q == 3 ? i + Q * l : p]) +
+                            X(c, 2, f)[Q == 3 ? i + Q * j : p];
+    ns_point<T>(v, gx, gy, gz, lap, F, P, c0, cxp, cyp, czp);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      U(c, f)[p] = c0[f];
+      G(c, 0, f)[p] = cxp[f];
+      G(c, 1, f)[p] = cyp[f];
+      G(c, 2, f)[p] = czp[f];
+    }
+  }
+  __syncthreads();
+  // ---- test side: transposed derivatives, then z, y, x
+  for (int it = tid; it < C * 12 * NL; it += 128) {
+    const int c = it / (12 * NL), d = it / (4 * NL) % 3, f = it / NL % 4, w = it % NL;
+    int p0, st;
+    line(d, w, p0, st);
+    T u[Q], o[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) u[a] = G(c, d, f)[p0 + st * a];
+    line_dwt<Q, false>(tab.Dw, tab.hDw, u, o);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) G(c, d, f)[p0 + st * a] = o[a];
+  }
+#pragma unroll
+  for (int dir = 2; dir >= 0; --dir) {
+    __syncthreads();
+    for (int it = tid; it < C * 4 * NL; it += 128) {
+      const int c = it / (4 * NL), f = it / NL % 4, w = it % NL;
+      int p0, st;
+      line(dir, w, p0, st);
+      T u[Q], o[Q];
+#pragma unroll
+      for (int a = 0; a < Q; ++a) {
+        const int p = p0 + st * a;
+        u[a] = U(c, f)[p];
+        if (dir == 2) u[a] = (u[a] + G(c, 0, f)[p]) + (G(c, 1, f)[p] + G(c, 2, f)[p]);
+      }
+      if (dir > 0) line_sym<Q, kTest, false>(tab.St, tab.hSt, u, o);
+      else if (f < 3) line_sym<Q, kTest, true>(tab.Sf, tab.hSf, u, o);
+      else line_sym<Q, kTest, true>(tab.Sfp, tab.hSfp, u, o);
+#pragma unroll
+      for (int a = 0; a < Q; ++a) U(c, f)[p0 + st * a] = o[a];
+    }
+  }
+  __syncthreads();
+  // ---- rows of node values; the face between x-neighbours of the block is added here
+  for (int it = tid; it < C * NP; it += 128) {
+    const int c = it / NP, p = it % NP, w = p / Q, a = p % Q;  // x-line w, node a
+    const uint32_t t = t0 + (uint32_t)c;
+    if (t >= P.cells) continue;
+    const int cx = (int)(t % (uint32_t)n), row = (int)(t / (uint32_t)n);
+    T r[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) r[f] = U(c, f)[p];
+    T* out = P.rows + (((int64_t)row * NL + w) * M + K * cx + a) * 4;
+    if (a == 0 && c > 0 && cx > 0)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) r[f] += U(c - 1, f)[p + K];
+    if (a == K && cx < n - 1) {
+      if (c < C - 1) continue;  // added by the neighbour
+      out = P.tails + ((int64_t)blk * NL + w) * 4;
+    }
+    *reinterpret_cast<double2*>(out) = make_double2(r[0], r[1]);
+    *reinterpret_cast<double2*>(out + 2) = make_double2(r[2], r[3]);
   }
 }
 
@@ -679,8 +864,8 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
       T o[Q];
-      if (f < 3) line_sym<Q, kTrial, false>(tab.S, val[f][b], o);
-      else line_sym<Q, kTrial, true>(tab.Sp, val[f][b], o);
+      if (f < 3) line_sym<Q, kTrial, false>(tab.S, tab.hS, val[f][b], o);
+      else line_sym<Q, kTrial, true>(tab.Sp, tab.hSp, val[f][b], o);
 #pragma unroll
       for (int a = 0; a < Q; ++a) val[f][b][a] = o[a];
     }
@@ -689,7 +874,7 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
       T u[Q], o[Q];
 #pragma unroll
       for (int b = 0; b < Q; ++b) u[b] = val[f][b][a];
-      line_sym<Q, kTrial, false>(tab.S, u, o);
+      line_sym<Q, kTrial, false>(tab.S, tab.hS, u, o);
 #pragma unroll
       for (int b = 0; b < Q; ++b) val[f][b][a] = o[b];
     }
@@ -735,8 +920,8 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
   for (int j = 0; j < Q; ++j) {
     T dx[4][Q], xx[4][Q], cxr[4][Q];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.D2, val[f][j], dx[f], xx[f]);
-    line_deriv<Q, false>(tab.D, tab.D2, val[3][j], dx[3], xx[3]);
+    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.hD, tab.D2, val[f][j], dx[f], xx[f]);
+    line_deriv<Q, false>(tab.D, tab.hD, tab.D2, val[3][j], dx[3], xx[3]);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       T F[4][4];
@@ -789,7 +974,7 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
       }
     }
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_dwt<Q, true>(tab.Dw, cxr[f], acc[f][j]);
+    for (int f = 0; f < 4; ++f) line_dwt<Q, true>(tab.Dw, tab.hDw, cxr[f], acc[f][j]);
   }
   __syncthreads();
   // ---- test side: z derivatives of the other planes, then the transposed values y, x and z
@@ -813,14 +998,14 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
       T u[Q], o[Q];
 #pragma unroll
       for (int j = 0; j < Q; ++j) u[j] = acc[f][j][i];
-      line_sym<Q, kTest, false>(tab.St, u, o);
+      line_sym<Q, kTest, false>(tab.St, tab.hSt, u, o);
 #pragma unroll
       for (int b = 0; b < Q; ++b) acc[f][b][i] = o[b];
     }
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
       T o[Q];
-      line_sym<Q, kTest, true>(f < 3 ? tab.Sf : tab.Sfp, acc[f][b], o);
+      line_sym<Q, kTest, true>(f < 3 ? tab.Sf : tab.Sfp, f < 3 ? tab.hSf : tab.hSfp, acc[f][b], o);
 #pragma unroll
       for (int a = 0; a < Q; ++a) acc[f][b][a] = o[a];
     }
@@ -935,7 +1120,7 @@ __global__ void __launch_bounds__(256) k_ns_nodes(const NsNodeArgs<T> a) {
       ld4(a.rows + ((row * NL + w) * M + ix) * 4, v[k]);
       if (face_x) {
         const uint32_t t = (uint32_t)row * (uint32_t)n + (uint32_t)qx;
-        const uint32_t blk = __umulhi(t, a.magic);
+        const uint32_t blk = a.C == 1 ? t : __umulhi(t, a.magic);
         cut[k] = blk * (uint32_t)a.C == t;
         if (cut[k]) ld4(a.tails + ((int64_t)(blk - 1) * NL + w) * 4, tl[k]);
       }

@@ -16,9 +16,8 @@ int ns_cells_per_block(int k, int prec, int64_t cells);
 size_t ns_fq_bytes(const OpLaunch& L, int prec);
 size_t ns_rows_bytes(const OpLaunch& L, int prec);
 
-// whether the cells run on the plane kernel (FP32 levels of full blocks) or on the line kernel; the
-// two round differently, and a multi-problem launch is of one kind
-bool ns_planes(int prec, int C);
+// the level's cell kernel (0, 1 or 2); they round differently, and a multi-problem launch is of one kind
+int ns_kernel(const OpLaunch& L, int prec);
 // blocks of a cell launch
 int64_t ns_blocks(const OpLaunch& L, int prec);
 // appends the descriptor of L's product to those of a multi-problem launch
