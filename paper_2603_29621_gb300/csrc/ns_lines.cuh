@@ -808,7 +808,9 @@ template <int K>
 struct NsPlane {
   static constexpr int Q = K + 1, NL = Q * Q, THREADS = 32 * Q;
   static constexpr int MINB = Q == 2 ? 8 : Q == 3 ? 5 : 2;
-  static constexpr size_t SMEM = 2 * (size_t)NL * Q * 32 * 16;
+  static constexpr int RING = Q == 3 ? 2 : 4;  // points of a thread's plane on their way (shared memory allows)
+  static constexpr size_t BUF = (size_t)NL * Q * 32 * 16;
+  static constexpr size_t SMEM = 2 * BUF + (size_t)RING * 4 * THREADS * 16;
 };
 
 template <int K, bool MULTI>
@@ -832,6 +834,23 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
     const unsigned bytes = (unsigned)(NL * Q * 64) * (unsigned)C;
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(fqb), "r"(bytes) : "memory");
   }
+  // ... and of this thread's first points into its slots of the ring (read back by the same thread)
+  constexpr int RING = NsPlane<K>::RING, NT = NsPlane<K>::THREADS;
+  const int fl = lane < C ? lane : C - 1;
+  const float4* fp = reinterpret_cast<const float4*>(fqb) + (int64_t)l * 4 * C + fl;
+  const float4* ring = reinterpret_cast<const float4*>(ns_smem + 2 * NsPlane<K>::BUF) + threadIdx.x;
+  const unsigned ring_s = (unsigned)__cvta_generic_to_shared(ring);
+  auto fetch = [&](int pt) {  // a group per point, empty past the last one
+    if (pt < NL)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(ring_s + (unsigned)((pt % RING * 4 + q) * NT * 16)),
+                     "l"(fp + ((int64_t)pt * Q * 4 + q) * C)
+                     : "memory");
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+#pragma unroll
+  for (int pt = 0; pt < RING; ++pt) fetch(pt);
   const uint32_t t = (uint32_t)blk * (uint32_t)C + (uint32_t)lane;
   const bool valid = lane < C && t < P.cells;
   const uint32_t tt = t < P.cells ? t : P.cells - 1;
@@ -911,11 +930,6 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
     for (int j = 0; j < Q; ++j)
 #pragma unroll
       for (int i = 0; i < Q; ++i) acc[f][j][i] = T(0);
-  const int fl = lane < C ? lane : C - 1;
-  const float4* fp = reinterpret_cast<const float4*>(fqb) + (int64_t)l * 4 * C + fl;
-  float4 Fn[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) Fn[q] = __ldg(fp + q * C);
 #pragma unroll
   for (int j = 0; j < Q; ++j) {
     T dx[4][Q], xx[4][Q], cxr[4][Q];
@@ -925,14 +939,11 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       T F[4][4];
+      asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 1) : "memory");
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        F[q][0] = Fn[q].x; F[q][1] = Fn[q].y; F[q][2] = Fn[q].z; F[q][3] = Fn[q].w;
-      }
-      if (i + Q * j + 1 < NL) {
-        fp += (int64_t)Q * 4 * C;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) Fn[q] = __ldg(fp + q * C);
+        const float4 v4 = ring[((i + Q * j) % RING * 4 + q) * NT];
+        F[q][0] = v4.x; F[q][1] = v4.y; F[q][2] = v4.z; F[q][3] = v4.w;
       }
       T gx[4], gy[4], gz[4], v[4], lap[3], c0[4], cxp[4], cyp[4], czp[4];
 #pragma unroll
@@ -963,6 +974,7 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
           for (int f = 0; f < 3; ++f) lap[f] = fma(d2, e[f], lap[f]);
       }
       ns_point<T>(v, gx, gy, gz, lap, F, P, c0, cxp, cyp, czp);
+      fetch(i + Q * j + RING);  // into the slots just read
       ns_st(Z, NL * l + i + Q * j, lane, 32, czp[0], czp[1], czp[2], czp[3]);
       const T dl = tab.Dw[l][l];
 #pragma unroll
