@@ -62,6 +62,8 @@ static void fill_ns(MultiOp& m, Budget* bud) {
 template <typename T>
 static void fill(MultiOp& m, Budget* bud) {
   if (m.L0->lq[m.prec]) return fill_ns(m, bud);
+  // (a member beyond the deferred products' bound would round differently alone and in a batch)
+  if (std::all_of(m.lv.begin(), m.lv.end(), [&](const OpLevel* l) { return l->gather && l->gather->tensor; })) return;
   const OpLaunch& L0 = *m.L0;
   const int nmem = (int)m.lv.size();
   const int ncol = L0.n_colors;
@@ -138,6 +140,11 @@ MultiOp* multi_op_create(const std::vector<const OpLevel*>& lv, const std::vecto
 
 // dst_i = A_i src_i for every member (constrained rows dst = src), one launch per colour.
 void multi_vmult(const MultiOp& m, cudaStream_t s) {
+  if (m.col.empty() && !m.ns[0].blocks && !m.ns[1].blocks && !m.ns[2].blocks) {
+    // tensor-product cells: one cell launch and node pass per member
+    for (size_t i = 0; i < m.lv.size(); ++i) oplevel_vmult(*m.lv[i], m.prec, m.src[i], m.dst[i], s);
+    return;
+  }
   if (m.ns[0].blocks || m.ns[1].blocks || m.ns[2].blocks) {
     for (const NsMulti& part : m.ns)
       if (part.blocks) ns_cells_multi(*m.L0, m.prec, part, s);

@@ -11,16 +11,26 @@
 
 namespace mfns {
 
-// Contributions of a level's nodes: entry e of node g (ptr[g] <= e < ptr[g + 1]) is slot idx[e] =
-// (cell position) * slots + slot, ascending, so a node's cells are added in colour order.
+// Contributions of a level's nodes: entries e of node g (ptr[g] <= e < ptr[g + 1]) are the places idx[e]
+// in the buffer, ascending.  Place of (cell, slot): position * slots + slot with cells in colour order,
+// so that a node's cells are added in that order; with tensor-product cells (`tensor`) slot * cells +
+// cell in the forest's order, so that neighbouring cells lie next to each other.
 struct NodeGather {
+  bool tensor = false;
+  int64_t cell_stride = 0, slot_stride = 0, cell_stride_p = 0, slot_stride_p = 0;
+  DevBuf pos;           // position of every cell of the colour order (transfers), or null: the same
+  // tensor-product cells: node per (slot, cell) with bit 31 on Dirichlet nodes, masks, edge lengths
+  DevBuf cell_u, cell_p, cell_mask, cell_h[2];
   DevBuf ptr, idx;      // main nodes
   DevBuf ptr_p, idx_p;  // Taylor--Hood pressure nodes
   DevBuf mask;          // per node (main, then pressure): bit f set where entry f is an identity row
   int64_t n_main = 0, n_p = 0, slots = 0, slots_p = 0;  // nodes; contributions of all cells
   int nu = 1;
   DevBuf buf[2];        // the contributions per precision: main, then pressure
-  size_t bytes() const { return ptr.bytes() + idx.bytes() + ptr_p.bytes() + idx_p.bytes() + mask.bytes() + buf[0].bytes() + buf[1].bytes(); }
+  size_t bytes() const {
+    return ptr.bytes() + idx.bytes() + ptr_p.bytes() + idx_p.bytes() + mask.bytes() + pos.bytes() + cell_u.bytes() + cell_p.bytes() +
+           cell_mask.bytes() + cell_h[0].bytes() + cell_h[1].bytes() + buf[0].bytes() + buf[1].bytes();
+  }
   int64_t main_values() const;  // values of the main part of buf
 };
 

@@ -7,6 +7,7 @@
 
 #include "ns_lines.hpp"
 #include "problem.hpp"
+#include "tensor_cells.hpp"
 #include "vec.hpp"
 
 namespace mfns {
@@ -273,7 +274,8 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
   }
   if (op != OP_VMASS && !lv.L.lq[0])
     for (int prec = 0; prec < 2; ++prec) {
-      lv.deferred[prec] = gather_fits(lv) && (!lv.L.structured || (int64_t)lv.L.n_cells <= kDeferMaxCells);
+      lv.deferred[prec] = gather_fits(lv) && (tensor_cells(lv.L) || !lv.L.structured ||
+                                              (int64_t)lv.L.n_cells <= kDeferMaxCells);
       if (lv.deferred[prec]) ensure_gather(lv, prec, bud);
     }
   lv.n_hang = (int64_t)hd.size();
@@ -286,7 +288,7 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
   lv.pres = upload(bud, lv.pres_host);
 }
 
-// contributions of slot lists: node ids of every (cell position, slot), bit 31 ignored
+// node tables: nodes[e] is the node of place e (bit 31 ignored)
 static void gather_table(const std::vector<int32_t>& nodes, int64_t n, std::vector<int32_t>& ptr,
                          std::vector<int32_t>& idx) {
   ptr.assign((size_t)n + 1, 0);
@@ -314,18 +316,37 @@ void ensure_gather(OpLevel& lv, int prec, Budget* bud) {
       G->n_p = lv.np.n_nodes;
       G->slots_p = (int64_t)nc * lv.np.nb;
     }
+    G->tensor = tensor_cells(lv.L);
     std::vector<int32_t> ptr, idx;
-    auto slots = [&](const NodeSpace& sp) {  // masters in the colour order of the cell tables
+    auto places = [&](const NodeSpace& sp, bool flag) {  // masters by place
       std::vector<int32_t> v(nc * sp.nb);
       for (size_t i = 0; i < nc; ++i)
-        for (int b = 0; b < sp.nb; ++b) v[i * sp.nb + b] = sp.cell_master[(size_t)lv.perm[i] * sp.nb + b];
+        for (int b = 0; b < sp.nb; ++b) {
+          const size_t c = G->tensor ? i : (size_t)lv.perm[i];
+          int32_t g = sp.cell_master[c * sp.nb + b];
+          if (flag && lv.op != OP_PMASS && sp.boundary[g]) g |= int32_t(0x80000000u);
+          v[G->tensor ? (size_t)b * nc + i : i * sp.nb + b] = g;
+        }
       return v;
     };
-    gather_table(slots(lv.nu), G->n_main, ptr, idx);
+    G->cell_stride = G->tensor ? 1 : lv.nu.nb;
+    G->slot_stride = G->tensor ? (int64_t)nc : 1;
+    if (G->tensor) {
+      G->pos = upload(bud, lv.perm);
+      G->cell_u = upload(bud, places(lv.nu, true));
+      const std::vector<uint32_t> masks = constraint_masks(lv.forest, make_lattice(lv.forest));
+      std::vector<double> h(nc);
+      for (size_t c = 0; c < nc; ++c) h[c] = lv.forest.h(c);
+      G->cell_mask = upload(bud, masks);
+      G->cell_h[0] = upload_as<double>(bud, h);
+      G->cell_h[1] = upload_as<float>(bud, h);
+      if (th) G->cell_p = upload(bud, places(lv.np, false));
+    }
+    gather_table(places(lv.nu, false), G->n_main, ptr, idx);
     G->ptr = upload(bud, ptr);
     G->idx = upload(bud, idx);
     if (th) {
-      gather_table(slots(lv.np), G->n_p, ptr, idx);
+      gather_table(places(lv.np, false), G->n_p, ptr, idx);
       G->ptr_p = upload(bud, ptr);
       G->idx_p = upload(bud, idx);
     }
@@ -349,7 +370,10 @@ static void node_product(const OpLevel& lv, int prec, const NsAfterArgs& a, cuda
     return;
   }
   const NodeGather& G = *lv.gather;
-  op_apply_deferred(lv.L, prec, a.src, G.buf[prec].get(), G.main_values(), s);
+  if (G.tensor)
+    tensor_product(lv.L, G, prec, a.src, s);
+  else
+    op_apply_deferred(lv.L, prec, a.src, G.buf[prec].get(), G.main_values(), s);
   gather_nodes(G, prec, a, s);
 }
 

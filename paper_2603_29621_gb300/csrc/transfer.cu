@@ -41,6 +41,8 @@ struct TransferArgs {
   int32_t cell_begin, cell_end;
   int hkind;
   T* defer;                   // restriction: contributions per (coarse cell, slot), or null: added into dst
+  const int32_t* pos;         // place of (cell, slot): position * cell_stride + slot * slot_stride
+  int64_t cell_stride, slot_stride;
 };
 
 // out = (Mz x My x Mx) in, matrices per direction selected by `sel` (0/1 half, 2 identity).
@@ -228,7 +230,8 @@ __global__ void __launch_bounds__(128) transfer_kernel(const TransferArgs<T, NF,
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const int slot = DIM == 3 ? (c * NC + tj) * NC + ti : c * NC + ti;
-        T* out = a.defer + (cell * NBC + slot) * defer_stride(NCOMP);
+        const int64_t at = (a.pos ? a.pos[cell] : cell) * a.cell_stride + slot * a.slot_stride;
+        T* out = a.defer + at * defer_stride(NCOMP);
 #pragma unroll
         for (int f = 0; f < NCOMP; ++f) {
           if (a.defer) out[f] = acc[f][c];
@@ -372,6 +375,9 @@ static void launch_transfer(const Transfer& t, const OpLevel& fine, const OpLeve
   }
   if (coarse.gather) {  // every coarse cell in one launch; transfer_restrict gathers
     a.defer = coarse.gather->buf[sizeof(T) == 8 ? 0 : 1].template as<T>();
+    a.pos = coarse.gather->pos.template as<int32_t>();
+    a.cell_stride = coarse.gather->cell_stride;
+    a.slot_stride = coarse.gather->slot_stride;
     a.cell_begin = 0;
     a.cell_end = (int32_t)t.n_coarse_cells;
     const unsigned grid = (unsigned)((t.n_coarse_cells + 4 * CPW - 1) / (4 * CPW));
