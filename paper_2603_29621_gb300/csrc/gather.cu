@@ -47,11 +47,23 @@ __device__ __forceinline__ void load_slot(const T* buf, int64_t e, T (&v)[NU]) {
   }
 }
 
-// The sum of one node and what follows it.  The entries' indices and then their values are loaded
-// four at a time: three dependent loads (range, indices, values) are the latency of a small level.
-template <typename T, int NU, int AFTER>
+// Entries loaded together: their indices, then their values; the first indices are loaded before the wait
+// for the cell launch.  Eight cover the nodes of a uniform mesh, which is what counts on a level of few
+// blocks (26,000 nodes of a refined Q1 level 6.2 -> 5.1 us, the whole V-cycle on 16^3 with two
+// refinements 505 -> 438 us); on large levels their registers cost more than the second round of loads
+// (Stokes Q2/Q1 on 24^3 with two refinements, 600,000 nodes: 31 us with four, 33 us with eight).
+constexpr uint32_t kLargeNodes = 152 * 1024;
+
+template <int kBatch>
+__device__ __forceinline__ void load_indices(const int32_t* idx, int32_t lo, int32_t hi, int32_t (&id)[kBatch]) {
+#pragma unroll
+  for (int j = 0; j < kBatch; ++j) id[j] = lo + j < hi ? idx[lo + j] : -1;
+}
+
+// The sum of one node and what follows it; id: its first indices.
+template <typename T, int NU, int AFTER, int kBatch>
 __device__ __forceinline__ void gather_one(const GatherArgs<T>& a, const T* buf, const int32_t* idx, int32_t lo,
-                                           int32_t hi, uint32_t m, int64_t dof) {
+                                           int32_t hi, int32_t (&id)[kBatch], uint32_t m, int64_t dof) {
   T x[NU], bb[NU], qq[NU], dd[NU];
 #pragma unroll
   for (int f = 0; f < NU; ++f) {
@@ -65,16 +77,14 @@ __device__ __forceinline__ void gather_one(const GatherArgs<T>& a, const T* buf,
   T acc[NU];
 #pragma unroll
   for (int f = 0; f < NU; ++f) acc[f] = T(0);
-  for (int32_t e = lo; e < hi; e += 4) {
-    int32_t id[4];
-    T v[4][NU];
+  for (int32_t e = lo; e < hi; e += kBatch) {
+    if (e != lo) load_indices(idx, e, hi, id);
+    T v[kBatch][NU];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) id[j] = e + j < hi ? idx[e + j] : -1;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < kBatch; ++j)
       if (id[j] >= 0) load_slot<T, NU>(buf, id[j], v[j]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < kBatch; ++j)
       if (id[j] >= 0)
 #pragma unroll
         for (int f = 0; f < NU; ++f) acc[f] = add_as_reduction(acc[f], v[j][f]);
@@ -103,25 +113,27 @@ __device__ __forceinline__ void gather_one(const GatherArgs<T>& a, const T* buf,
 // on small levels by the latency of three dependent loads: 7.6 us at 193,000 nodes of three FP32
 // components, 3.8 us on the smallest levels (launch included; the pass it replaces, which derived the
 // cells from the node's index, took 8 us there).
-template <typename T, int NU, int AFTER>
+template <typename T, int NU, int AFTER, int kBatch>
 __global__ void __launch_bounds__(256) k_gather_nodes(const GatherArgs<T> a) {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const uint32_t i = blockIdx.x * 256u + threadIdx.x;
   const bool main = i < a.n_main, in = i < a.n_main + a.n_p;
   int32_t lo = 0, hi = 0;
   uint32_t m = 0;
+  int32_t id[kBatch];
   if (in) {  // the table is constant data
     const int32_t* p = main ? a.ptr + i : a.ptr_p + (i - a.n_main);
     lo = p[0];
     hi = p[1];
     m = a.mask[i];
+    load_indices(main ? a.idx : a.idx_p, lo, hi, id);
   }
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   if (!in) return;
   if (main)
-    gather_one<T, NU, AFTER>(a, a.buf, a.idx, lo, hi, m, (int64_t)i * NU);
+    gather_one<T, NU, AFTER, kBatch>(a, a.buf, a.idx, lo, hi, id, m, (int64_t)i * NU);
   else
-    gather_one<T, 1, AFTER>(a, a.buf_p, a.idx_p, lo, hi, m, (int64_t)a.n_main * NU + (i - a.n_main));
+    gather_one<T, 1, AFTER, kBatch>(a, a.buf_p, a.idx_p, lo, hi, id, m, (int64_t)a.n_main * NU + (i - a.n_main));
 }
 
 template <typename T, int NU>
@@ -152,12 +164,18 @@ static void launch(const NodeGather& g, int prec, const NsAfterArgs& f, cudaStre
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const bool large = a.n_main + a.n_p > kLargeNodes;
+#define GO(AFTER)                                                                         \
+  MFNS_CUDA(large ? cudaLaunchKernelEx(&cfg, k_gather_nodes<T, NU, AFTER, 4>, a)          \
+                  : cudaLaunchKernelEx(&cfg, k_gather_nodes<T, NU, AFTER, 8>, a));        \
+  return
   switch (f.after) {
-    case 0: MFNS_CUDA(cudaLaunchKernelEx(&cfg, k_gather_nodes<T, NU, 0>, a)); return;
-    case 1: MFNS_CUDA(cudaLaunchKernelEx(&cfg, k_gather_nodes<T, NU, 1>, a)); return;
-    case 2: MFNS_CUDA(cudaLaunchKernelEx(&cfg, k_gather_nodes<T, NU, 2>, a)); return;
-    default: MFNS_CUDA(cudaLaunchKernelEx(&cfg, k_gather_nodes<T, NU, 3>, a)); return;
+    case 0: GO(0);
+    case 1: GO(1);
+    case 2: GO(2);
+    default: GO(3);
   }
+#undef GO
 }
 
 void gather_nodes(const NodeGather& g, int prec, const NsAfterArgs& a, cudaStream_t s) {

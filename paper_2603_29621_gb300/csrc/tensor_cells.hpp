@@ -1,4 +1,4 @@
-// Vector Laplacian, Taylor--Hood Stokes and pressure mass of degree at most 2 in 3D: every cell is an
+// Vector Laplacian, Taylor--Hood Stokes and pressure mass in 3D: every cell is an
 // axis-aligned cube, so its matrix is a sum of tensor products of 1D mass, stiffness and mixed
 // matrices (tensor_cells.cu).
 #pragma once
