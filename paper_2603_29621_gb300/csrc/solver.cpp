@@ -301,9 +301,10 @@ void alloc_workspaces(Problem& p) {
   p.tmp.alloc(bud, n * 8);
   p.sys_r.alloc(bud, n * 8);
   p.sys_z.alloc(bud, n * 8);
-  p.hvec.alloc(bud, 2 * kMaxDots * 8);
+  p.hvec.alloc(bud, (2 * kMaxDots + 1) * 8);
   p.yvec.alloc(bud, kMaxDots * 8);
-  p.part.alloc(bud, (size_t)kRedBlocks * kMaxDots * 8);
+  p.part.alloc(bud, (size_t)kRedScratch * 8);
+  MFNS_CUDA(cudaMemset(p.part.get(), 0, (size_t)kRedScratch * 8));
   p.scal.alloc(bud, 16 * 8);
   std::vector<const double*> pv(m + 1), pz(m);
   for (int j = 0; j <= m; ++j) pv[j] = p.V.as<double>() + (size_t)j * n;
@@ -505,10 +506,11 @@ double arnoldi_spectral_radius(Problem& p, OpLevel& lv, cudaStream_t s,
     else
       vmul<double>(w, dinv, p.tmp.as<double>(), n, s);
     double* hd = p.hvec.as<double>();
-    multidot(hd, nullptr, w, j + 1, n, p.part.as<double>(), Vp, s);
-    multi_axpy(w, Vp, hd, j + 1, n, s);
-    multidot(hd + kMaxDots, nullptr, w, j + 1, n, p.part.as<double>(), Vp, s);
-    multi_axpy(w, Vp, hd + kMaxDots, j + 1, n, s);
+    double* part = p.part.as<double>();
+    multidot(hd, w, j + 1, n, part, Vp, s);
+    multi_axpy(w, Vp, hd, j + 1, n, nullptr, part, s);
+    multidot(hd + kMaxDots, w, j + 1, n, part, Vp, s);
+    multi_axpy(w, Vp, hd + kMaxDots, j + 1, n, nullptr, part, s);
     std::vector<double> hh(2 * kMaxDots);
     MFNS_CUDA(cudaMemcpyAsync(hh.data(), hd, 2 * kMaxDots * 8, cudaMemcpyDeviceToHost, s));
     const double hn = std::sqrt(host_dot(p, w, w, n, s));
@@ -879,25 +881,45 @@ static void stokes_block(Problem& p, int prec, const T* r, T* z, cudaStream_t s)
 
 static void precondition_body(Problem& p, const double* v, double* z, cudaStream_t s);
 
+// The multigrid cycle (Eq. 5: the block preconditioner) between fixed buffers of precision T
+template <typename T>
+static void precondition_core(Problem& p, const T* b, T* x, cudaStream_t s) {
+  if (p.kind == 0)
+    stokes_block<T>(p, sizeof(T) == 4, b, x, s);
+  else
+    mg_cycle<T>(p, sizeof(T) == 4, b, x, s);
+}
+
 // The preconditioner is a fixed sequence of kernels on fixed buffers: it is captured once into
-// a CUDA graph (input p.pc_in, output p.pc_out) and replayed.
+// a CUDA graph (FP64: p.pc_in to p.pc_out; FP32: p.mg_b32 to p.mg_x32) and replayed between the copies,
+// or conversions, of its input and output.
 static void precondition(Problem& p, const double* v, double* z, cudaStream_t s) {
   OpLevel& S = p.system ? *p.system : *p.levels[0];
   const int64_t n = S.n_dofs;
   if (!p.use_graphs) return precondition_body(p, v, z, s);
+  const bool fp32 = p.mg_precision == 1;
   if (!p.pc_graph) {
     if (!p.cap_stream) MFNS_CUDA(cudaStreamCreateWithFlags(&p.cap_stream, cudaStreamNonBlocking));
     TimerPause pause(p);
     MFNS_CUDA(cudaStreamBeginCapture(p.cap_stream, cudaStreamCaptureModeThreadLocal));
-    precondition_body(p, p.pc_in.as<double>(), p.pc_out.as<double>(), p.cap_stream);
+    if (fp32)
+      precondition_core<float>(p, p.mg_b32.as<float>(), p.mg_x32.as<float>(), p.cap_stream);
+    else
+      precondition_core<double>(p, p.pc_in.as<double>(), p.pc_out.as<double>(), p.cap_stream);
     cudaGraph_t g;
     MFNS_CUDA(cudaStreamEndCapture(p.cap_stream, &g));
     MFNS_CUDA(cudaGraphInstantiate(&p.pc_graph, g, 0));
     MFNS_CUDA(cudaGraphDestroy(g));
   }
-  MFNS_CUDA(cudaMemcpyAsync(p.pc_in.get(), v, n * 8, cudaMemcpyDeviceToDevice, s));
+  if (fp32)
+    vcast_d2f(p.mg_b32.as<float>(), v, n, s);
+  else
+    MFNS_CUDA(cudaMemcpyAsync(p.pc_in.get(), v, n * 8, cudaMemcpyDeviceToDevice, s));
   MFNS_CUDA(cudaGraphLaunch(p.pc_graph, s));
-  MFNS_CUDA(cudaMemcpyAsync(z, p.pc_out.get(), n * 8, cudaMemcpyDeviceToDevice, s));
+  if (fp32)
+    vcast_f2d(z, p.mg_x32.as<float>(), n, s);
+  else
+    MFNS_CUDA(cudaMemcpyAsync(z, p.pc_out.get(), n * 8, cudaMemcpyDeviceToDevice, s));
 }
 
 void invalidate_graphs(Problem& p) {
@@ -930,19 +952,12 @@ void vcycle_graph(Problem& p, int prec, const void* b, void* x, cudaStream_t s) 
 }
 
 static void precondition_body(Problem& p, const double* v, double* z, cudaStream_t s) {
-  OpLevel& S = sys_of(p);
-  const int64_t n = S.n_dofs;
+  const int64_t n = sys_of(p).n_dofs;
   if (p.mg_precision == 0) {
-    if (p.kind == 0)
-      stokes_block<double>(p, 0, v, z, s);
-    else
-      mg_cycle<double>(p, 0, v, z, s);
+    precondition_core<double>(p, v, z, s);
   } else {
     vcast_d2f(p.mg_b32.as<float>(), v, n, s);
-    if (p.kind == 0)
-      stokes_block<float>(p, 1, p.mg_b32.as<float>(), p.mg_x32.as<float>(), s);
-    else
-      mg_cycle<float>(p, 1, p.mg_b32.as<float>(), p.mg_x32.as<float>(), s);
+    precondition_core<float>(p, p.mg_b32.as<float>(), p.mg_x32.as<float>(), s);
     vcast_f2d(z, p.mg_x32.as<float>(), n, s);
   }
 }
@@ -956,8 +971,7 @@ static void start_cycle(Problem& p, double beta) {
   OpLevel& S = sys_of(p);
   Krylov& K = p.kry;
   const int m = p.restart;
-  vcopy<double>(p.V.as<double>(), p.tmp.as<double>(), S.n_dofs, K.stream);
-  vscale<double>(p.V.as<double>(), 1.0 / beta, S.n_dofs, K.stream);
+  vscale_copy(p.V.as<double>(), 1.0 / beta, p.tmp.as<double>(), S.n_dofs, K.stream);
   std::fill(K.g.begin(), K.g.end(), 0.0);
   K.g[0] = beta;
   K.j = 0;
@@ -1041,13 +1055,12 @@ static void krylov_after_precondition(Problem& p, double* zj) {
   project_pressure<double>(S, zj, p.scal.as<double>(), p.part.as<double>(), s);
   oplevel_vmult(S, 0, zj, w, s);
   double* hd = p.hvec.as<double>();
-  multidot(hd, nullptr, w, j + 1, n, p.part.as<double>(), Vp, s);
-  multi_axpy(w, Vp, hd, j + 1, n, s);
-  multidot(hd + kMaxDots, nullptr, w, j + 1, n, p.part.as<double>(), Vp, s);
-  multi_axpy(w, Vp, hd + kMaxDots, j + 1, n, s);
-  dot<double>(p.scal.as<double>() + 12, w, w, n, p.part.as<double>(), s);
-  MFNS_CUDA(cudaMemcpyAsync(p.hh_host, hd, 2 * kMaxDots * 8, cudaMemcpyDeviceToHost, s));
-  MFNS_CUDA(cudaMemcpyAsync(p.hh_host + 2 * kMaxDots, p.scal.as<double>() + 12, 8, cudaMemcpyDeviceToHost, s));
+  double* part = p.part.as<double>();
+  multidot(hd, w, j + 1, n, part, Vp, s);
+  multi_axpy(w, Vp, hd, j + 1, n, nullptr, part, s);
+  multidot(hd + kMaxDots, w, j + 1, n, part, Vp, s);
+  multi_axpy(w, Vp, hd + kMaxDots, j + 1, n, hd + 2 * kMaxDots, part, s);
+  MFNS_CUDA(cudaMemcpyAsync(p.hh_host, hd, (2 * kMaxDots + 1) * 8, cudaMemcpyDeviceToHost, s));
 }
 
 // Host part of the step (after the problem's stream has been synchronised); ends the restart
@@ -1067,8 +1080,7 @@ bool krylov_complete(Problem& p) {
   for (int i = 0; i <= j; ++i) H[i * m + j] = hh[i] + hh[kMaxDots + i];
   H[(j + 1) * m + j] = hn;
   if (hn > 0) {
-    vcopy<double>(V + (size_t)(j + 1) * n, p.w.as<double>(), n, s);
-    vscale<double>(V + (size_t)(j + 1) * n, 1.0 / hn, n, s);
+    vscale_copy(V + (size_t)(j + 1) * n, 1.0 / hn, p.w.as<double>(), n, s);
   }
   for (int i = 0; i < j; ++i) {
     const double t = K.cs[i] * H[i * m + j] + K.sn[i] * H[(i + 1) * m + j];

@@ -658,11 +658,10 @@ static int stmg_fgmres(mfns_spacetime& st, const double* b, double* x, double to
       // one multi-axpy, and one host round trip per iteration for both passes and the norm
       const double** Vp = (const double**)mg.ptrV.as<const double*>();
       double* hd = mg.hvec.as<double>();
-      multidot(hd, nullptr, w, j + 1, N, mg.part.as<double>(), Vp, s);
-      multi_axpy(w, Vp, hd, j + 1, N, s);
-      multidot(hd + kMaxDots, nullptr, w, j + 1, N, mg.part.as<double>(), Vp, s);
-      multi_axpy(w, Vp, hd + kMaxDots, j + 1, N, s);
-      dot<double>(hd + 2 * kMaxDots, w, w, N, mg.part.as<double>(), s);
+      multidot(hd, w, j + 1, N, mg.part.as<double>(), Vp, s);
+      multi_axpy(w, Vp, hd, j + 1, N, nullptr, mg.part.as<double>(), s);
+      multidot(hd + kMaxDots, w, j + 1, N, mg.part.as<double>(), Vp, s);
+      multi_axpy(w, Vp, hd + kMaxDots, j + 1, N, hd + 2 * kMaxDots, mg.part.as<double>(), s);
       MFNS_CUDA(cudaMemcpyAsync(mg.hh_host, hd, (size_t)(2 * kMaxDots + 1) * 8, cudaMemcpyDeviceToHost, s));
       MFNS_CUDA(cudaStreamSynchronize(s));
       for (int i = 0; i <= j; ++i) {
@@ -673,8 +672,7 @@ static int stmg_fgmres(mfns_spacetime& st, const double* b, double* x, double to
       const double hn = std::sqrt(std::max(mg.hh_host[2 * kMaxDots], 0.0));
       H[(size_t)(j + 1) * m + j] = hn;
       if (hn > 0.0) {
-        MFNS_CUDA(cudaMemcpyAsync(V + (int64_t)(j + 1) * N, w, (size_t)N * 8, cudaMemcpyDeviceToDevice, s));
-        vscale<double>(V + (int64_t)(j + 1) * N, 1.0 / hn, N, s);
+        vscale_copy(V + (int64_t)(j + 1) * N, 1.0 / hn, w, N, s);
       }
       for (int i = 0; i < j; ++i) {  // earlier rotations
         const double a = H[(size_t)i * m + j], c = H[(size_t)(i + 1) * m + j];
@@ -828,7 +826,8 @@ static void build_stmg(mfns_spacetime& st, int nu_s, double omega, int coarse_n,
   mg->cn = N;
   mg->pres = upload(bud, pres);
   mg->n_pres = (int64_t)pres.size();
-  mg->part.alloc(bud, (size_t)kRedBlocks * kMaxDots * 8);
+  mg->part.alloc(bud, (size_t)kRedScratch * 8);
+  MFNS_CUDA(cudaMemset(mg->part.get(), 0, (size_t)kRedScratch * 8));
   mg->scal.alloc(bud, 64);
   const std::vector<int32_t> pres0 = pressure_entries(*mg->lv[0]);
   mg->pres0 = upload(bud, pres0);

@@ -22,6 +22,7 @@ template <typename T> __global__ void k_axpby(T* y, T a, const T* x, T b, int64_
 }
 template <typename T> __global__ void k_sub(T* r, const T* b, const T* ax, int64_t n) { GRID_STRIDE(i, n) r[i] = b[i] - ax[i]; }
 template <typename T> __global__ void k_scale(T* y, T a, int64_t n) { GRID_STRIDE(i, n) y[i] *= a; }
+__global__ void k_scale_copy(double* y, double a, const double* x, int64_t n) { GRID_STRIDE(i, n) y[i] = a * x[i]; }
 __global__ void k_d2f(float* y, const double* x, int64_t n) { GRID_STRIDE(i, n) y[i] = (float)x[i]; }
 __global__ void k_unit_cols(double* X, int64_t n, int64_t j0, int64_t nb) {
   GRID_STRIDE(t, n * nb) {
@@ -141,65 +142,120 @@ template <typename T> __global__ void k_gemv(T* y, const T* M, const T* x, int64
   if (lane == 0) y[row] = (T)s;
 }
 
-// block reduction of kRedThreads doubles
-__device__ double block_sum(double v, double* sh) {
-  sh[threadIdx.x] = v;
+// Sums over the grid in one launch: every block writes its partial sums, the block that finishes last adds
+// them in block order (a fixed grid and order: deterministic) and resets the counter behind the
+// partial sums.  sh: the warps' sums.  Bound by launches and FP64 additions at the sizes of a solve: the
+// eight multi-dots, updates, dots and their separate final sums of an iteration took 95 us at 276,000
+// entries, these five launches 45 us (20^3 Q2Q2 solve 4.66 -> 4.34 ms).
+constexpr int kRedWarps = kRedThreads / 32;
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ void finish_sums(double (&sh)[kRedWarps][kMaxDots], int m, double* part, double* out) {
+  __shared__ bool last;
+  unsigned* counter = reinterpret_cast<unsigned*>(part + (size_t)kRedBlocks * kMaxDots);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nb = (int)gridDim.x;
   __syncthreads();
-  for (int o = kRedThreads / 2; o; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
+  if ((int)threadIdx.x < m) {
+    double s = 0;
+#pragma unroll
+    for (int w = 0; w < kRedWarps; ++w) s += sh[w][threadIdx.x];
+    part[(size_t)threadIdx.x * nb + blockIdx.x] = s;
+    __threadfence();
   }
-  double r = sh[0];
   __syncthreads();
-  return r;
+  if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int k = warp; k < m; k += kRedWarps) {
+    double s = 0;
+    for (int i = lane; i < nb; i += 32) s += __ldcg(part + (size_t)k * nb + i);
+    s = warp_sum(s);
+    if (lane == 0) out[k] = s;
+  }
+  if (threadIdx.x == 0) *counter = 0;
 }
 
-__global__ void k_multidot_part(double* part, const double* const* V, const double* w, int m, int64_t n) {
-  __shared__ double sh[kRedThreads];
-  for (int k = 0; k < m; ++k) {
-    double s = 0;
-    const double* v = V[k];
-    for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads)
-      s += v[i] * w[i];
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) part[k * gridDim.x + blockIdx.x] = s;
+// out[k] = sum_i V_k[i] w[i]: eight products per pass over w
+__global__ void __launch_bounds__(kRedThreads) k_multidot(double* out, double* part, const double* const* V,
+                                                          const double* w, int m, int64_t n) {
+  __shared__ double sh[kRedWarps][kMaxDots];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int k0 = 0; k0 < m; k0 += 8) {
+    const double* v[8];
+    double acc[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v[k] = V[k0 + k < m ? k0 + k : k0];
+      acc[k] = 0;
+    }
+    for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads) {
+      const double wi = w[i];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k0 + k < m) acc[k] += v[k][i] * wi;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (k0 + k >= m) break;
+      const double s = warp_sum(acc[k]);
+      if (lane == 0) sh[warp][k0 + k] = s;
+    }
   }
+  finish_sums(sh, m, part, out);
 }
-__global__ void k_final(double* out, const double* part, int m, int nb) {
-  __shared__ double sh[kRedThreads];
-  for (int k = 0; k < m; ++k) {
-    double s = 0;
-    for (int i = threadIdx.x; i < nb; i += kRedThreads) s += part[k * nb + i];
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) out[k] = s;
-  }
-}
-template <typename T> __global__ void k_dot_part(double* part, const T* a, const T* b, int64_t n) {
-  __shared__ double sh[kRedThreads];
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) k_dot(double* out, double* part, const T* a, const T* b, int64_t n) {
+  __shared__ double sh[kRedWarps][kMaxDots];
   double s = 0;
   for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads)
     s += (double)a[i] * (double)b[i];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][0] = s;
+  finish_sums(sh, 1, part, out);
 }
-template <typename T> __global__ void k_sum_idx_part(double* part, const T* x, const int32_t* idx, int64_t n) {
-  __shared__ double sh[kRedThreads];
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) k_sum_idx(double* out, double* part, const T* x, const int32_t* idx,
+                                                         int64_t n) {
+  __shared__ double sh[kRedWarps][kMaxDots];
   double s = 0;
   for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads)
     s += (double)x[idx[i]];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][0] = s;
+  finish_sums(sh, 1, part, out);
+}
+// w -= sum_k h[k] V_k and, with norm2, *norm2 = sum of the new w^2
+__global__ void __launch_bounds__(kRedThreads) k_multi_axpy(double* w, const double* const* V, const double* h, int m,
+                                                            int64_t n, double* norm2, double* part) {
+  __shared__ double sh[kRedWarps][kMaxDots];
+  __shared__ double hs[kMaxDots];
+  __shared__ const double* vs[kMaxDots];
+  if ((int)threadIdx.x < m) {
+    hs[threadIdx.x] = h[threadIdx.x];
+    vs[threadIdx.x] = V[threadIdx.x];
+  }
+  __syncthreads();
+  double nn = 0;
+  for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads) {
+    double s = w[i];
+#pragma unroll 4
+    for (int k = 0; k < m; ++k) s -= hs[k] * vs[k][i];
+    w[i] = s;
+    nn += s * s;
+  }
+  if (!norm2) return;
+  nn = warp_sum(nn);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][0] = nn;
+  finish_sums(sh, 1, part, norm2);
 }
 template <typename T> __global__ void k_sub_mean_idx(T* x, const int32_t* idx, int64_t n, const double* sum) {
   const T mean = (T)(*sum / (double)n);
   GRID_STRIDE(i, n) x[idx[i]] -= mean;
-}
-__global__ void k_multi_axpy(double* w, const double* const* V, const double* h, int m, int64_t n) {
-  GRID_STRIDE(i, n) {
-    double s = w[i];
-    for (int k = 0; k < m; ++k) s -= h[k] * V[k][i];
-    w[i] = s;
-  }
 }
 __global__ void k_multi_axpy_add(double* x, const double* const* Z, const double* y, int m, int64_t n) {
   GRID_STRIDE(i, n) {
@@ -313,30 +369,25 @@ template <typename T> void vgemv(T* y, const T* M, const T* x, int64_t n, cudaSt
   MFNS_CUDA(cudaGetLastError());
 }
 
-void multidot(double* out, const double* const* V, const double* w, int m, int64_t n, double* part,
-              const double** Vdev, cudaStream_t s) {
-  (void)V;
-  k_multidot_part<<<kRedBlocks, kRedThreads, 0, s>>>(part, Vdev, w, m, n);
-  MFNS_CUDA(cudaGetLastError());
-  k_final<<<1, kRedThreads, 0, s>>>(out, part, m, kRedBlocks);
+void multidot(double* out, const double* w, int m, int64_t n, double* part, const double* const* Vdev, cudaStream_t s) {
+  k_multidot<<<kRedBlocks, kRedThreads, 0, s>>>(out, part, Vdev, w, m, n);
   MFNS_CUDA(cudaGetLastError());
 }
 template <typename T> void dot(double* out, const T* a, const T* b, int64_t n, double* part, cudaStream_t s) {
-  k_dot_part<T><<<kRedBlocks, kRedThreads, 0, s>>>(part, a, b, n);
-  MFNS_CUDA(cudaGetLastError());
-  k_final<<<1, kRedThreads, 0, s>>>(out, part, 1, kRedBlocks);
+  k_dot<T><<<kRedBlocks, kRedThreads, 0, s>>>(out, part, a, b, n);
   MFNS_CUDA(cudaGetLastError());
 }
-void multi_axpy(double* w, const double* const* Vdev, const double* h, int m, int64_t n, cudaStream_t s) {
-  LAUNCH(k_multi_axpy, n, s, w, Vdev, h, m, n);
+void multi_axpy(double* w, const double* const* Vdev, const double* h, int m, int64_t n, double* norm2, double* part,
+                cudaStream_t s) {
+  k_multi_axpy<<<kRedBlocks, kRedThreads, 0, s>>>(w, Vdev, h, m, n, norm2, part);
+  MFNS_CUDA(cudaGetLastError());
 }
 void multi_axpy_add(double* x, const double* const* Zdev, const double* y, int m, int64_t n, cudaStream_t s) {
   LAUNCH(k_multi_axpy_add, n, s, x, Zdev, y, m, n);
 }
+void vscale_copy(double* y, double a, const double* x, int64_t n, cudaStream_t s) { LAUNCH(k_scale_copy, n, s, y, a, x, n); }
 template <typename T> void sum_idx(double* out, const T* x, const int32_t* idx, int64_t n, double* part, cudaStream_t s) {
-  k_sum_idx_part<T><<<kRedBlocks, kRedThreads, 0, s>>>(part, x, idx, n);
-  MFNS_CUDA(cudaGetLastError());
-  k_final<<<1, kRedThreads, 0, s>>>(out, part, 1, kRedBlocks);
+  k_sum_idx<T><<<kRedBlocks, kRedThreads, 0, s>>>(out, part, x, idx, n);
   MFNS_CUDA(cudaGetLastError());
 }
 template <typename T> void sub_mean_idx(T* x, const int32_t* idx, int64_t n, const double* sum, cudaStream_t s) {

@@ -68,13 +68,18 @@ template <typename T> void vrecip(T* y, const T* x, int64_t n, cudaStream_t s);
 // dense gemv y = M x (row-major n x n)
 template <typename T> void vgemv(T* y, const T* M, const T* x, int64_t n, cudaStream_t s);
 
-// Deterministic reductions into device scratch `part` (kRedBlocks * kMaxDots doubles) and
-// the final result `out` (device, double): out[k] = sum_i V_k[i] w[i], k < m.
-void multidot(double* out, const double* const* V, const double* w, int m, int64_t n, double* part,
-              const double** Vdev, cudaStream_t s);
+// y = a x
+void vscale_copy(double* y, double a, const double* x, int64_t n, cudaStream_t s);
+
+// Deterministic reductions, one launch each, through device scratch `part` of kRedScratch doubles that is
+// zeroed once (its last double holds the counter by which the last block recognises itself; a scratch
+// serves one stream at a time).  out[k] = sum_i V_k[i] w[i], k < m (device, double).
+constexpr int kRedScratch = kRedBlocks * kMaxDots + 1;
+void multidot(double* out, const double* w, int m, int64_t n, double* part, const double* const* Vdev, cudaStream_t s);
 template <typename T> void dot(double* out, const T* a, const T* b, int64_t n, double* part, cudaStream_t s);
-// w -= sum_k h[k] V_k (h on device)
-void multi_axpy(double* w, const double* const* Vdev, const double* h, int m, int64_t n, cudaStream_t s);
+// w -= sum_k h[k] V_k (h on device); *norm2 (device, may be null) = sum of the new w^2
+void multi_axpy(double* w, const double* const* Vdev, const double* h, int m, int64_t n, double* norm2, double* part,
+                cudaStream_t s);
 // x += sum_k y[k] Z_k (y on device)
 void multi_axpy_add(double* x, const double* const* Zdev, const double* y, int m, int64_t n, cudaStream_t s);
 // sum of x over idx (device double result)
