@@ -12,6 +12,7 @@
 // ten cells a warp; tables are uniform operands and index lists are stored by slot, so their loads are
 // consecutive over cells.  Bound by instruction issue and the latency of the gather.
 #include <atomic>
+#include <type_traits>
 
 #include "common.hpp"
 #include "op_kernel.cuh"
@@ -343,10 +344,10 @@ __global__ void __launch_bounds__(128) k_tensor_cells(const __grid_constant__ Tp
 // A component's (k + 1)^3 values no longer fit a thread: a thread owns one line of one component, and the
 // fields go through shared memory between the directions, three stages and two barriers (six more in a
 // block with hanging nodes).  FP64 products are bound by the number of operations.
-template <int N, int NP, int KIND>
+template <int N, int NP, int KIND, int TH>
 struct TpLines {
   static constexpr int NL = N * N, NB = NL * N, NBP = NP * NP * NP, COMP = KIND == 2 ? 1 : 3;
-  static constexpr int C = 256 / (COMP * NL);
+  static constexpr int C = TH / (COMP * NL);
   // per cell: A, B [COMP][NB]; Stokes: W [3][NP N N], T1, T2 [NP NP N], P0, P1 [NP NP N], P00, P01, P10 [NP N N]
   static constexpr int oB = COMP * NB, oW = KIND == 2 ? oB : 2 * oB, oT = oW + 3 * NP * NL, oP = oT + 2 * NP * NP * N,
                        oPP = oP + 2 * NP * NP * N, CELL = KIND == 1 ? oPP + 3 * NP * NL : oW;
@@ -391,9 +392,9 @@ __device__ __forceinline__ bool line_hangs(uint32_t m, int dir, int w) {
   return dir == 0 ? LineFlags<3, N>::x(m, p, q) : dir == 1 ? LineFlags<3, N>::y(m, p, q) : LineFlags<3, N>::z(m, p, q);
 }
 
-template <int N, int NP, int KIND, typename T>
-__global__ void __launch_bounds__(256, 3) k_tensor_lines(const __grid_constant__ TpArgs<T, N, NP> a) {
-  using Tl = TpLines<N, NP, KIND>;
+template <int N, int NP, int KIND, int TH, typename T>
+__global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_constant__ TpArgs<T, N, NP> a) {
+  using Tl = TpLines<N, NP, KIND, TH>;
   constexpr int NL = Tl::NL, NB = Tl::NB, NPL = NP * NP, COMP = Tl::COMP, C = Tl::C, CELL = Tl::CELL;
   constexpr int OUT = defer_stride(COMP);
   extern __shared__ __align__(16) unsigned char tp_smem[];
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(256, 3) k_tensor_lines(const __grid_constant__
   if (any) {  // resolve the hanging nodes first: velocity into A, pressure into P00
     for (int dir = 0; dir < 3; ++dir) {
       if (dir) __syncthreads();
-      for (int it = threadIdx.x; it < vel; it += 256) {
+      for (int it = threadIdx.x; it < vel; it += TH) {
         const int c = it / (COMP * NL), f = it / NL % COMP, w = it % NL;
         const uint32_t m = a.mask[c0 + c];
         int p0, st;
@@ -431,7 +432,7 @@ __global__ void __launch_bounds__(256, 3) k_tensor_lines(const __grid_constant__
         for (int i = 0; i < N; ++i) A[p0 + st * i] = v[i];
       }
       if constexpr (KIND == 1)
-        for (int it = threadIdx.x; it < ncell * NPL; it += 256) {
+        for (int it = threadIdx.x; it < ncell * NPL; it += TH) {
           const int c = it / NPL, w = it % NPL;
           const uint32_t m = a.mask[c0 + c];
           int p0, st;
@@ -711,28 +712,41 @@ static void launch(const OpLaunch& L, const NodeGather& g, int prec, const void*
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if constexpr (N <= 3) {
+  // (FP64 starts on an idle chip, see ns_lines.cu)
+  if (sizeof(T) == 8) cfg.numAttrs = 0;
+  auto lines = [&](auto th) {
+    constexpr int TH = decltype(th)::value;
+    using Tl = TpLines<N, NP, KIND, TH>;
+    constexpr size_t smem = (size_t)Tl::C * Tl::CELL * sizeof(T);
+    if (smem > 48 * 1024) {
+      static std::atomic<uint64_t> done{0};  // per device
+      int dev = 0;
+      MFNS_CUDA(cudaGetDevice(&dev));
+      const uint64_t bit = 1ull << (dev & 63);
+      if (!(done.load() & bit)) {
+        MFNS_CUDA(cudaFuncSetAttribute(k_tensor_lines<N, NP, KIND, TH, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem));
+        done.fetch_or(bit);
+      }
+    }
+    cfg.gridDim = dim3((unsigned)((L.n_cells + Tl::C - 1) / Tl::C));
+    cfg.blockDim = dim3(TH);
+    cfg.dynamicSmemBytes = smem;
+    MFNS_CUDA(cudaLaunchKernelEx(&cfg, k_tensor_lines<N, NP, KIND, TH, T>, a));
+  };
+  if constexpr (N > 3) {
+    lines(std::integral_constant<int, 256>());
+  } else if constexpr (sizeof(T) == 8) {
+    // FP64: a warp's operations take 64 cycles each, so a cell's lines go to many lanes (Q2 Stokes in registers
+    // 37 us from 4^3 to 16^3 cells, lines 14 to 31 us); the smaller blocks spread further, the larger
+    // ones waste fewer lanes and are the better ones from two a SM on (Q2 48^3 379 against 421 us)
+    if (KIND != 2 && L.n_cells >= 2 * 152 * (256 / (3 * N * N))) lines(std::integral_constant<int, 256>());
+    else lines(std::integral_constant<int, 128>());
+  } else {
     constexpr int per_block = 4 * (KIND == 2 ? 32 : 10);
     cfg.gridDim = dim3((unsigned)((L.n_cells + per_block - 1) / per_block));
     cfg.blockDim = dim3(128);
     MFNS_CUDA(cudaLaunchKernelEx(&cfg, k_tensor_cells<N, NP, KIND, T>, a));
-  } else {
-    using Tl = TpLines<N, NP, KIND>;
-    constexpr size_t smem = (size_t)Tl::C * Tl::CELL * sizeof(T);
-    static std::atomic<uint64_t> done{0};  // per device
-    int dev = 0;
-    MFNS_CUDA(cudaGetDevice(&dev));
-    const uint64_t bit = 1ull << (dev & 63);
-    if (!(done.load() & bit)) {
-      MFNS_CUDA(cudaFuncSetAttribute(k_tensor_lines<N, NP, KIND, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      done.fetch_or(bit);
-    }
-    cfg.gridDim = dim3((unsigned)((L.n_cells + Tl::C - 1) / Tl::C));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = smem;
-    // (FP64 on an idle chip, see ns_lines.cu)
-    if (sizeof(T) == 8) cfg.numAttrs = 0;
-    MFNS_CUDA(cudaLaunchKernelEx(&cfg, k_tensor_lines<N, NP, KIND, T>, a));
   }
   if (timed) L.timer->record_pair_end(s);
 }
