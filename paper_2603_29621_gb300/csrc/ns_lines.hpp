@@ -48,4 +48,7 @@ struct NsAfterArgs {
 };
 void ns_nodes(const OpLaunch& L, int prec, const NsAfterArgs& a, void* rows, cudaStream_t s);
 
+// diagonal with 1 on the identity rows; rows: the level's row buffer (scratch)
+void ns_diagonal(const OpLaunch& L, int prec, void* diag, void* rows, cudaStream_t s);
+
 }  // namespace mfns

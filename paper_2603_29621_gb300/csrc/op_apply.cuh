@@ -53,12 +53,6 @@ template <int DIM, int K, int OP, typename T>
 struct OpMinBlocks {
   static constexpr int value = 1;
 };
-// the diagonal of a uniform 3D stabilised level keeps the frozen state's point values in registers
-// through its unit-vector passes (no staged blocks there): no occupancy bound
-template <int DIM, int K, int OP, typename T, bool DIAG, int FQ>
-constexpr int op_min_blocks() {
-  return DIAG && FQ == 0 ? 1 : OpMinBlocks<DIM, K, OP, T>::value;
-}
 #ifndef MFNS_STABNS_Q2_F32_MINBLOCKS
 #define MFNS_STABNS_Q2_F32_MINBLOCKS 6
 #endif
@@ -137,7 +131,7 @@ template <int DIM, int K, int OP, typename T, bool STRUCT, bool DIAG, int FQ = 0
           bool MULTI = false, bool DEFER = false>
 __global__ void __launch_bounds__(kOpWarps * 32, (EPI && OpMinBlocks<DIM, K, OP, T>::value > 1)
                                                      ? OpMinBlocks<DIM, K, OP, T>::value - 1
-                                                     : op_min_blocks<DIM, K, OP, T, DIAG, FQ>())
+                                                     : OpMinBlocks<DIM, K, OP, T>::value)
 op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
   constexpr int Q = K + 1, N = K + 1, NP = OP == OP_STOKES ? K : K + 1;
   using Tr = OpTraits<OP, DIM>;
@@ -146,6 +140,9 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
   constexpr int NB = ipow(N, DIM);
   constexpr int NBP = ipow(NP, DIM);
   constexpr int BUF = TM::BUF;
+  // one launch over every colour (structured: blockIdx.y): deferred products and the set-up pass,
+  // whose cells write entries of their own
+  constexpr bool ALL = DEFER || FQ == 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* smem = reinterpret_cast<T*>(smem_raw);
   // per-problem fields: kernel parameters, or the descriptor of the problem owning this block
@@ -176,13 +173,13 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
 #pragma unroll
     for (int i = 0; i < 7; ++i) cf_[i] = pa->cf[i];
   } else {
-    srcp = args.src + (DEFER ? 0 : (int64_t)blockIdx.y * args.col_stride);
-    dstp = args.dst + (DEFER ? 0 : (int64_t)blockIdx.y * args.col_stride);
+    srcp = args.src + (ALL ? 0 : (int64_t)blockIdx.y * args.col_stride);
+    dstp = args.dst + (ALL ? 0 : (int64_t)blockIdx.y * args.col_stride);
     frozen = args.frozen;
     gexp = args.gexp;
     fqd = args.fq;
     nmesh = args.n;
-    color_offset = DEFER ? args.defer_off[blockIdx.y] : args.color_offset;
+    color_offset = ALL ? args.defer_off[blockIdx.y] : args.color_offset;
     p_offset = args.p_offset;
     bx = (int64_t)blockIdx.x;
     hs = args.h;
@@ -227,13 +224,13 @@ op_kernel(const OpArgs<T, K + 1, K + 1, (OP == OP_STOKES ? K : K + 1)> args) {
       int m[3], bits[3];
       int64_t total = 1;
       for (int d = 0; d < 3; ++d) {
-        bits[d] = d < DIM ? ((DEFER ? (int)blockIdx.y : args.color) >> d) & 1 : 0;
+        bits[d] = d < DIM ? ((ALL ? (int)blockIdx.y : args.color) >> d) & 1 : 0;
         m[d] = d < DIM ? (n - bits[d] + 1) / 2 : 1;
         total *= m[d];
       }
-      // a deferred launch spans all colours, some of which may hold no cell (n = 1): such a
+      // a launch that spans all colours, some of which may hold no cell (n = 1): such a
       // colour's blocks leave before touching memory (total is uniform over the block)
-      if (DEFER && total == 0) return;
+      if (ALL && total == 0) return;
       valid = lane_active && t < total;
       const int64_t tt = t < total ? t : total - 1;
       cc[0] = 2 * (int)(tt % m[0]) + bits[0];

@@ -76,6 +76,29 @@ static void fill_common(const OpLaunch& L, OpArgs<T, Q, N, NP>& a) {
   a.gexp = reinterpret_cast<const T*>(L.gexp[prec]);
 }
 
+// Grid and colour offsets of a launch over every cell (structured: blockIdx.y = colour).
+template <int DIM, typename Args>
+static dim3 grid_of_all(const OpLaunch& L, int cells_per_block, Args& a) {
+  int64_t maxc = L.n_cells;
+  unsigned gy = 1;
+  if (L.structured) {
+    gy = 1u << DIM;
+    int64_t off = 0;
+    maxc = 0;
+    for (unsigned c = 0; c < gy; ++c) {
+      int64_t nc = 1;
+      for (int d = 0; d < DIM; ++d) nc *= (L.n - ((c >> d) & 1) + 1) / 2;
+      a.defer_off[c] = off;
+      off += nc;
+      maxc = std::max(maxc, nc);
+    }
+  } else {
+    a.cell_begin = 0;
+    a.cell_end = (int32_t)L.n_cells;
+  }
+  return dim3((unsigned)((maxc + cells_per_block - 1) / cells_per_block), gy);
+}
+
 template <int DIM, int K, int OP, typename T>
 void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t s, int fq_mode, int ncols,
                int64_t col_stride, const OpEpilogue* epi) {
@@ -137,6 +160,16 @@ void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t 
       attr_done.fetch_or(bit);
     }
   }
+  if constexpr (OP == OP_STAB_NS)
+    if (fq == 2) {  // set-up pass: every cell at once
+      const dim3 grid = grid_of_all<DIM>(L, cells_per_block, a);
+      if (L.structured)
+        op_kernel<DIM, K, OP, T, true, false, 2><<<grid, warps * 32, smem, s>>>(a);
+      else
+        op_kernel<DIM, K, OP, T, false, false, 2><<<grid, warps * 32, smem, s>>>(a);
+      MFNS_CUDA(cudaGetLastError());
+      return;
+    }
   const bool structured = L.structured && !diag;
   int64_t color_offset = 0;
   bool launched = epi && epi->after_clear;  // the clearing kernel before colour 0 lets it start early
@@ -175,12 +208,7 @@ void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t 
     launched = true;
     auto go = [&](auto kern, size_t sm) { launch_op(kern, grid, warps * 32, sm, s, a, pdl); };
     if constexpr (OP == OP_STAB_NS) {
-      if (fq == 2) {
-        if (L.structured)
-          go(op_kernel<DIM, K, OP, T, true, false, 2>, smem);
-        else
-          go(op_kernel<DIM, K, OP, T, false, false, 2>, smem);
-      } else if (fq == 3) {
+      if (fq == 3) {
         if (L.structured)
           go(op_kernel<DIM, K, OP, T, true, false, 3>, smem);
         else
@@ -238,24 +266,7 @@ void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, T* defer_p, c
   const int prec = sizeof(T) == 8 ? 0 : 1;
   const int warps = L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
   const int cells_per_block = warps * TM::CPW;
-  int64_t maxc = L.n_cells;
-  unsigned gy = 1;
-  if (L.structured) {
-    gy = 1u << DIM;
-    int64_t off = 0;
-    maxc = 0;
-    for (unsigned c = 0; c < gy; ++c) {
-      int64_t nc = 1;
-      for (int d = 0; d < DIM; ++d) nc *= (L.n - ((c >> d) & 1) + 1) / 2;
-      a.defer_off[c] = off;
-      off += nc;
-      maxc = std::max(maxc, nc);
-    }
-  } else {
-    a.cell_begin = 0;
-    a.cell_end = (int32_t)L.n_cells;
-  }
-  const dim3 grid((unsigned)((maxc + cells_per_block - 1) / cells_per_block), gy);
+  const dim3 grid = grid_of_all<DIM>(L, cells_per_block, a);
   const bool timed = L.timer && L.timer->enabled;
   if (timed) L.timer->record_pair_begin(s);
   auto go = [&](auto kern, size_t sm) { launch_op(kern, grid, warps * 32, sm, s, a, true); };

@@ -196,6 +196,7 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
       // uniform 3D levels: the layout of ns_lines.cuh, and the rows through which a product is summed
       for (int prec = 0; prec < 2; ++prec) {
         L.lc[prec] = ns_cells_per_block(k, prec, (int64_t)nc);
+        L.warps[prec] = 1;  // of the general kernel (residual, diagonal, set-up): spread over the chip
         lv.fq[prec].alloc(bud, ns_fq_bytes(L, prec));
         lv.rows[prec].alloc(bud, ns_rows_bytes(L, prec));
         // spare slots of the last block hold zeros; the tails that no block writes are not read
@@ -474,6 +475,7 @@ void oplevel_residual_fused(const OpLevel& lv, int prec, const void* x, const vo
 
 void oplevel_diag(const OpLevel& lv, int prec, void* diag, cudaStream_t s) {
   if (lv.hp) return hp_diag(lv, prec, diag, s);
+  if (lv.L.lq[prec]) return ns_diagonal(lv.L, prec, diag, lv.rows[prec].get(), s);
   MFNS_CUDA(cudaMemsetAsync(diag, 0, lv.n_dofs * esize(prec), s));
   op_apply(lv.L, prec, nullptr, diag, true, s);
   const int64_t nc = (int64_t)lv.constrained_host.size();
