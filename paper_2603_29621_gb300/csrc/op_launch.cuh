@@ -264,12 +264,16 @@ void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, T* defer_p, c
   a.defer_p = defer_p;
   using TM = Team<DIM, Q>;
   const int prec = sizeof(T) == 8 ? 0 : 1;
-  const int warps = L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
+  // FP64: one-warp blocks, spread over as many SMs as there are (the tuned size is that of colour launches)
+  const int warps = sizeof(T) == 8 ? 1 : L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
   const int cells_per_block = warps * TM::CPW;
   const dim3 grid = grid_of_all<DIM>(L, cells_per_block, a);
   const bool timed = L.timer && L.timer->enabled;
   if (timed) L.timer->record_pair_begin(s);
-  auto go = [&](auto kern, size_t sm) { launch_op(kern, grid, warps * 32, sm, s, a, true); };
+  // FP64 products of more than a few blocks start on an idle chip: started early, the blocks pile up on the
+  // first SMs that are free (2D NS Q2 64 x 64 cells 68 us against 25; 16 x 16 cells, 28 blocks: 21 against 25 us)
+  const bool pdl = sizeof(T) == 4 || grid.x * grid.y <= 152 / 4;
+  auto go = [&](auto kern, size_t sm) { launch_op(kern, grid, warps * 32, sm, s, a, pdl); };
   bool staged = false;
   if constexpr (OP == OP_STAB_NS) {
     staged = a.fq != nullptr;  // point values staged per cell (2D and refined levels)

@@ -12,15 +12,21 @@
 
 namespace mfns {
 
-// Which products are deferred (one cell launch and a node pass) instead of one launch per colour: every
-// locally refined level (its 17 to 30 colours were most of a product: Stokes Q2/Q1, 24^3 cells with
-// two refinements, FP32 110 -> 70 us; the vector Laplacian's V-cycle on 16^3 with two refinements 1866 ->
-// 707 us), and uniform levels of at most this many cells (2D Stokes 16 x 16 FP64 19.6 -> 11.7 us; at
-// 24^3 Q3/Q2 FP64 the colours' launches are long enough to be the better ones, 341 against 352 us).
-#ifndef MFNS_DEFER_MAX_CELLS
-#define MFNS_DEFER_MAX_CELLS 4096
-#endif
-constexpr int64_t kDeferMaxCells = MFNS_DEFER_MAX_CELLS;
+// Which products are deferred (one cell launch and a node pass) instead of one launch per colour:
+// - every locally refined level (its 17 to 30 colours were most of a product: Stokes Q2/Q1, 24^3 cells with
+//   two refinements, FP32 110 -> 70 us; the vector Laplacian's V-cycle on 16^3 with two refinements
+//   1866 -> 707 us);
+// - 2D uniform levels up to 2^19 (FP64) or 2^20 (FP32) contributions, where the launches' latency and
+//   partly filled launches cost more than the contributions' way through memory (FP64 Stokes Q2 16^2
+//   19.6 -> 12.2 us, 128^2 73 -> 31 us, 320^2 (2^19.8) 154 and 154 us; NS Q3 128^2 129 -> 121 us, 192^2 (2^19.2)
+//   215 against 223 us; FP32 NS Q2 320^2 24 -> 22 us, Q3 320^2 (2^20.6) 35 against 36 us);
+// - 3D uniform levels without point values or tensor products, up to 4096 cells.
+constexpr int64_t kDeferMaxCells3 = 4096;
+constexpr int64_t kDeferMaxPlaces2[2] = {int64_t(1) << 19, int64_t(1) << 20};
+static bool defer_uniform(const OpLevel& lv, int prec) {
+  return lv.dim == 3 ? lv.L.n_cells <= kDeferMaxCells3
+                     : (int64_t)lv.L.n_cells * lv.nu.nb <= kDeferMaxPlaces2[prec];
+}
 constexpr int64_t kDeferMaxValues = int64_t(1) << 29;  // contributions of a level (4 GiB in FP64)
 
 size_t OpLevel::bytes() const {
@@ -275,8 +281,7 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
   }
   if (op != OP_VMASS && !lv.L.lq[0])
     for (int prec = 0; prec < 2; ++prec) {
-      lv.deferred[prec] = gather_fits(lv) && (tensor_cells(lv.L) || !lv.L.structured ||
-                                              (int64_t)lv.L.n_cells <= kDeferMaxCells);
+      lv.deferred[prec] = gather_fits(lv) && (tensor_cells(lv.L) || !lv.L.structured || defer_uniform(lv, prec));
       if (lv.deferred[prec]) ensure_gather(lv, prec, bud);
     }
   lv.n_hang = (int64_t)hd.size();
