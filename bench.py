@@ -30,7 +30,8 @@ sys.path.insert(0, ROOT)
 
 METRIC = "DoF/s stab-NS Q2 vmult; solves/s + p50/p99 latency, FP32-MG vs FP64 @1e-8"
 UNIT = "DoF/s"
-FLOP_PER_CELL = 17000.0          # algorithmic flops per Q2Q2 cell apply, frozen point values precomputed
+FLOP_PER_CELL = 8000.0           # flops per Q2Q2 cell apply: 4,600 operations, most of them FMAs (even-odd 1D
+                                 # products, factors folded into tables and point values)
 FQ_BYTES_PER_CELL_F32 = 16 * 27 * 4  # precomputed frozen point data read per cell (u, grad u, Rbar, tau)
 FP32_LANES, N_SM, SM_MHZ_MAX = 128, 152, 2070.0
 CPU_SAMPLE_N = 12                # oracle sample: 12^3 cells of the same operator
@@ -147,15 +148,15 @@ class Clocks:
 
 def kernel_src_hash():
     h = hashlib.sha256()
-    for f in ("op_apply.cuh", "op_kernel.cuh", "op_launch.cuh"):
+    for f in ("ns_lines.cuh", "ns_lines.cu"):
         h.update(open(os.path.join(ROOT, "paper_2603_29621_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
 
 def ncu_traffic():
-    """DRAM bytes per launch of the FP32 structured cell kernel from the committed ncu summary,
+    """DRAM bytes per launch of the FP32 cell kernel from the committed ncu summary,
     or None when the kernel sources changed since the capture."""
-    path = os.path.join(ROOT, "profiles", "op_kernel_stabns_q2_fp32.md")
+    path = os.path.join(ROOT, "profiles", "ns_product_q2_fp32.md")
     if not os.path.exists(path):
         return None
     vals = {}
@@ -870,15 +871,15 @@ def run_ours(args, world, rank, local):
         barrier()
         return total / steps  # ms per step
 
-    # ---- headline: FP32 vmult as a user runs it (later colours overlap the previous colour's tail)
+    # ---- headline: FP32 vmult as a user runs it (the node pass starts while the cell launch drains)
     # clocks sampled over the headline, the per-launch pass and the end-to-end passes (the headline
     # alone lasts a few milliseconds, shorter than the sampling period)
     clocks = Clocks(local)
     clocks.wait_ready()
     clocks.mark()
     ms32 = timed(lambda: prob.vmult(src32, dst32), args.steps, args.warmup, nvtx="timed_vmult_fp32")
-    # ---- the cell kernel's colour launches one by one, each bracketed by CUDA events on the
-    # launching stream (the events serialise the launches): the per-launch roofline figure
+    # ---- the cell kernel's launches, each bracketed by CUDA events on the launching stream (the
+    # events serialise the launches): the per-launch roofline figure
     prob.kernel_timing(1)
     timed(lambda: prob.vmult(src32, dst32), args.steps, args.warmup)
     kms, klaunch = prob.kernel_timing(2)
@@ -983,8 +984,8 @@ def run_ours(args, world, rank, local):
         pass
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     # algorithmic bytes of one apply: src and dst (4 fields each) and the frozen state (u, p: 4
-    # fields) once per node, FP32 -- 12 x 2,146,689 x 4 B = 103.0 MB at 64^3; a colour launch
-    # processes 1/launches_per_step of the cells and is charged that share
+    # fields) once per node, FP32 -- 12 x 2,146,689 x 4 B = 103.0 MB at 64^3; the cell launch
+    # processes all cells and is charged all of it
     alg_bytes = 12 * nodes * 4
     bytes_launch = alg_bytes * cells_per_launch / ncell
     achieved = bytes_launch / (avg_launch_ms * 1e-3) / 1e9
@@ -994,7 +995,7 @@ def run_ours(args, world, rank, local):
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": headline_config(n, world),
         "clocks": clk,
-        # per step: the clearing kernel (which also writes the identity rows) and the colour launches
+        # per step: the cell launch and the node pass
         "gpu_launches": (launches_per_step + 1) * args.steps,
         "e2e": {"value": whole_job_rate(ndof, world, ms_e2e), "unit": UNIT, "h2d_bytes_per_step": ndof * 4,
                 "d2h_bytes_per_step": ndof * 4, "ms_per_step": ms_e2e,
@@ -1007,12 +1008,12 @@ def run_ours(args, world, rank, local):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                      "frac": achieved / hbm_peak, "traffic": traffic,
                      "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy, burst), of measured",
-                     "kernel": "op_kernel<3,2,STAB_NS,float,structured> (one colour launch)",
+                     "kernel": "k_ns_planes<2> (the cell launch of a product)",
                      "alg_bytes_per_apply": alg_bytes, "alg_bytes_per_launch": bytes_launch,
                      "alg_bytes_rule": "12 fields (src 4, dst 4, frozen u,p 4) x nodes x 4 B",
                      "cells_per_launch": cells_per_launch, "avg_launch_ms": avg_launch_ms,
-                     "avg_launch_note": "launches timed one by one (events serialise them); in the "
-                                        "headline apply later colours overlap the previous colour's tail",
+                     "avg_launch_note": "cell launches timed by themselves (events serialise them); the "
+                                        "headline apply adds the node pass, which overlaps their tail",
                      "launches_per_apply": launches_per_step,
                      "whole_apply": {"achieved_gbs": alg_bytes / (ms32 * 1e-3) / 1e9,
                                      "frac": alg_bytes / (ms32 * 1e-3) / 1e9 / hbm_peak},
@@ -1021,8 +1022,8 @@ def run_ours(args, world, rank, local):
                              "peak_rule": "152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz"},
                      "ridge_flop_per_byte": peak_alu * 1e12 / (hbm_peak * 1e9),
                      "intensity_flop_per_byte": FLOP_PER_CELL * ncell / alg_bytes,
-                     "with_point_data": {"note": "bytes the kernel reads by design: src, dst and the "
-                                                 "precomputed frozen point block (1,728 B per cell)",
+                     "with_point_data": {"note": "bytes the product moves by design: src, dst and the "
+                                                 "precomputed point values (1,728 B per cell)",
                                          "bytes_per_launch": (8 * nodes * 4 * cells_per_launch / ncell
                                                               + cells_per_launch * FQ_BYTES_PER_CELL_F32),
                                          "achieved_gbs": (8 * nodes * 4 * cells_per_launch / ncell

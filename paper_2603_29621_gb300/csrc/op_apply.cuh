@@ -45,7 +45,7 @@ struct Team {
 
 // Minimum resident blocks per SM for the register allocator (occupancy vs spills), per
 // instantiation; 1 lets the compiler use up to 255 registers.  The 3D Q2 stabilised kernel in
-// FP32 (the headline product) runs best at 6 x 128 threads' worth (80 registers, 8 bytes of
+// FP32 (refined levels and levels without stored point values) runs best at 6 x 128 threads' worth (80 registers, 8 bytes of
 // spill): measured on the 64^3 apply, 4 / 5 / 6 / 7 / 8 gave 0.222 / 0.208 / 0.199 / 0.214 /
 // 0.232 ms (the latency of the late dst loads and the shared-memory exchanges wants warps).
 // The fused-epilogue instantiation gets one block less (its update operands need registers).

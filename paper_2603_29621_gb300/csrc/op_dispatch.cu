@@ -272,12 +272,9 @@ void op_apply_deferred(const OpLaunch& L, int prec, const void* src, void* defer
   if (L.dim == DIM && L.k == K && L.op == OP) return op_launch_deferred<DIM, K, OP, T>(L, x, d, dp, s);
     MFNS_CASE(3, 1, OP_STAB_NS) MFNS_CASE(3, 2, OP_STAB_NS) MFNS_CASE(3, 3, OP_STAB_NS)
     MFNS_CASE(2, 1, OP_STAB_NS) MFNS_CASE(2, 2, OP_STAB_NS) MFNS_CASE(2, 3, OP_STAB_NS) MFNS_CASE(2, 4, OP_STAB_NS)
-    MFNS_CASE(3, 2, OP_STOKES) MFNS_CASE(3, 3, OP_STOKES) MFNS_CASE(3, 4, OP_STOKES)
     MFNS_CASE(2, 2, OP_STOKES) MFNS_CASE(2, 3, OP_STOKES) MFNS_CASE(2, 4, OP_STOKES)
-    MFNS_CASE(3, 1, OP_STOKES_A) MFNS_CASE(3, 2, OP_STOKES_A) MFNS_CASE(3, 3, OP_STOKES_A) MFNS_CASE(3, 4, OP_STOKES_A)
     MFNS_CASE(2, 1, OP_STOKES_A) MFNS_CASE(2, 2, OP_STOKES_A) MFNS_CASE(2, 3, OP_STOKES_A) MFNS_CASE(2, 4, OP_STOKES_A)
     MFNS_CASE(2, 1, OP_PMASS) MFNS_CASE(2, 2, OP_PMASS) MFNS_CASE(2, 3, OP_PMASS)
-    MFNS_CASE(3, 1, OP_PMASS) MFNS_CASE(3, 2, OP_PMASS) MFNS_CASE(3, 3, OP_PMASS)
 #undef MFNS_CASE
     throw Error(kErrUnsupported, "deferred products: (dim, degree, operator)");
   };

@@ -256,58 +256,62 @@ void op_launch(const OpLaunch& L, const T* src, T* dst, bool diag, cudaStream_t 
 // contributions to `defer` (and `defer_p`); k_gather_nodes forms the product from them.
 template <int DIM, int K, int OP, typename T>
 void op_launch_deferred(const OpLaunch& L, const T* src, T* defer, T* defer_p, cudaStream_t s) {
-  constexpr int Q = K + 1, N = K + 1, NP = OP == OP_STOKES ? K : K + 1;
-  OpArgs<T, Q, N, NP> a{};
-  fill_common(L, a);
-  a.src = src;
-  a.defer = defer;
-  a.defer_p = defer_p;
-  using TM = Team<DIM, Q>;
-  const int prec = sizeof(T) == 8 ? 0 : 1;
-  // FP64: one-warp blocks, spread over as many SMs as there are (the tuned size is that of colour launches)
-  const int warps = sizeof(T) == 8 ? 1 : L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
-  const int cells_per_block = warps * TM::CPW;
-  const dim3 grid = grid_of_all<DIM>(L, cells_per_block, a);
-  const bool timed = L.timer && L.timer->enabled;
-  if (timed) L.timer->record_pair_begin(s);
-  // FP64 products of more than a few blocks start on an idle chip: started early, the blocks pile up on the
-  // first SMs that are free (2D NS Q2 64 x 64 cells 68 us against 25; 16 x 16 cells, 28 blocks: 21 against 25 us)
-  const bool pdl = sizeof(T) == 4 || grid.x * grid.y <= 152 / 4;
-  auto go = [&](auto kern, size_t sm) { launch_op(kern, grid, warps * 32, sm, s, a, pdl); };
-  bool staged = false;
-  if constexpr (OP == OP_STAB_NS) {
-    staged = a.fq != nullptr;  // point values staged per cell (2D and refined levels)
-    if (staged) {
-      const size_t sm = op_smem_bytes<DIM, K, OP, T>(warps, true);
-      static std::atomic<uint64_t> attr_done{0};  // per device, for the largest block size
-      int dev = 0;
-      MFNS_CUDA(cudaGetDevice(&dev));
-      const uint64_t bit = 1ull << (dev & 63);
-      if (!(attr_done.load() & bit)) {
-        const int mx = (int)op_smem_bytes<DIM, K, OP, T>(kOpWarps, true);
-        if constexpr (DIM == 2)
-          MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1, false, false, true>,
+  if constexpr (DIM == 3 && OP != OP_STAB_NS) {
+    throw Error(kErrUnsupported, "deferred products: 3D Stokes operators are tensor products (tensor_cells.cu)");
+  } else {
+    constexpr int Q = K + 1, N = K + 1, NP = OP == OP_STOKES ? K : K + 1;
+    OpArgs<T, Q, N, NP> a{};
+    fill_common(L, a);
+    a.src = src;
+    a.defer = defer;
+    a.defer_p = defer_p;
+    using TM = Team<DIM, Q>;
+    const int prec = sizeof(T) == 8 ? 0 : 1;
+    // FP64: one-warp blocks, spread over as many SMs as there are (the tuned size is that of colour launches)
+    const int warps = sizeof(T) == 8 ? 1 : L.warps[prec] > 0 ? L.warps[prec] : kOpWarps;
+    const int cells_per_block = warps * TM::CPW;
+    const dim3 grid = grid_of_all<DIM>(L, cells_per_block, a);
+    const bool timed = L.timer && L.timer->enabled;
+    if (timed) L.timer->record_pair_begin(s);
+    // FP64 products of more than a few blocks start on an idle chip: started early, the blocks pile up on the
+    // first SMs that are free (2D NS Q2 64 x 64 cells 68 us against 25; 16 x 16 cells, 28 blocks: 21 against 25 us)
+    const bool pdl = sizeof(T) == 4 || grid.x * grid.y <= 152 / 4;
+    auto go = [&](auto kern, size_t sm) { launch_op(kern, grid, warps * 32, sm, s, a, pdl); };
+    bool staged = false;
+    if constexpr (OP == OP_STAB_NS) {
+      staged = a.fq != nullptr;  // point values staged per cell (2D and refined levels)
+      if (staged) {
+        const size_t sm = op_smem_bytes<DIM, K, OP, T>(warps, true);
+        static std::atomic<uint64_t> attr_done{0};  // per device, for the largest block size
+        int dev = 0;
+        MFNS_CUDA(cudaGetDevice(&dev));
+        const uint64_t bit = 1ull << (dev & 63);
+        if (!(attr_done.load() & bit)) {
+          const int mx = (int)op_smem_bytes<DIM, K, OP, T>(kOpWarps, true);
+          if constexpr (DIM == 2)
+            MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, true, false, 1, false, false, true>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+          MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, false, false, 1, false, false, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        MFNS_CUDA(cudaFuncSetAttribute(op_kernel<DIM, K, OP, T, false, false, 1, false, false, true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        attr_done.fetch_or(bit);
+          attr_done.fetch_or(bit);
+        }
+        if (!L.structured)
+          go(op_kernel<DIM, K, OP, T, false, false, 1, false, false, true>, sm);
+        else if constexpr (DIM == 2)
+          go(op_kernel<DIM, K, OP, T, true, false, 1, false, false, true>, sm);
+        else
+          throw Error(kErrArg, "stored point values of a uniform 3D level: another layout");
       }
-      if (!L.structured)
-        go(op_kernel<DIM, K, OP, T, false, false, 1, false, false, true>, sm);
-      else if constexpr (DIM == 2)
-        go(op_kernel<DIM, K, OP, T, true, false, 1, false, false, true>, sm);
-      else
-        throw Error(kErrArg, "stored point values of a uniform 3D level: another layout");
     }
+    if (!staged) {
+      const size_t sm = op_smem_bytes<DIM, K, OP, T>(warps, false);
+      if (L.structured)
+        go(op_kernel<DIM, K, OP, T, true, false, 0, false, false, true>, sm);
+      else
+        go(op_kernel<DIM, K, OP, T, false, false, 0, false, false, true>, sm);
+    }
+    if (timed) L.timer->record_pair_end(s);
   }
-  if (!staged) {
-    const size_t sm = op_smem_bytes<DIM, K, OP, T>(warps, false);
-    if (L.structured)
-      go(op_kernel<DIM, K, OP, T, true, false, 0, false, false, true>, sm);
-    else
-      go(op_kernel<DIM, K, OP, T, false, false, 0, false, false, true>, sm);
-  }
-  if (timed) L.timer->record_pair_end(s);
 }
 
 template <int DIM, int K, int OP, typename T>
