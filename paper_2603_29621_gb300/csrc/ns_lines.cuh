@@ -23,9 +23,9 @@
 // and for several in a launch.
 //
 // Measured against eight colour launches of the warp-per-three-cells kernel (whole product, GB300): Q2
-// 64^3 FP32 176 -> 129 us, 48^3 FP64 1849 -> 1114 us (FP64 pipe 87 % busy), Q3 31^3 FP32 61.8 -> 60.1 us,
-// five Q1 45^3 FP32 smoothing sweeps 116 -> 52 us.  The FP32 cell launch (103 us at 64^3) is bound by
-// the DRAM stream of the point values (5.4 TB/s), the node pass (28 us) by its rows.
+// 64^3 FP32 176 -> 119 us, 48^3 FP64 1849 -> 1116 us (FP64 pipe 87 % busy), Q3 31^3 FP32 61.8 -> 58 us,
+// five Q1 45^3 FP32 smoothing sweeps 116 -> 50 us.  The FP32 cell launch (95 us at 64^3) is bound by
+// the DRAM stream of the point values (5.7 TB/s), the node pass (about 25 us) by its rows.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -1101,7 +1101,8 @@ struct NsNodeArgs {
 };
 
 // Node pass: bound by the reads of `rows` (L2-resident up to 64^3 in FP32) and the vectors.  One
-// thread per node; the (at most four) rows of a node are loaded together.
+// thread per node; the (at most four) rows of a node are loaded together.  (Two nodes per thread: 64^3
+// FP32 product 119 -> 135 us; registers bounded for six or eight blocks a SM: 133, 140 us.)
 template <typename T, int K, int AFTER>
 __global__ void __launch_bounds__(256) k_ns_nodes(const NsNodeArgs<T> a) {
   constexpr int Q = K + 1, NL = Q * Q;
@@ -1159,7 +1160,9 @@ __global__ void __launch_bounds__(256) k_ns_nodes(const NsNodeArgs<T> a) {
   }
   T sum[4];
   T x4[4], b4[4], q4[4], d4[4];
-  ld4(a.src + node * 4, x4);
+  // the source only where it is used: the iterate, or identity rows (64^3 FP32 product 123.2 -> 118.7 us)
+  const bool bnd = ix == 0 || ix == M - 1 || iy == 0 || iy == M - 1 || iz == 0 || iz == M - 1;
+  if (AFTER == kUpdate || bnd) ld4(a.src + node * 4, x4);
   if constexpr (AFTER != kStore) ld4(a.b + node * 4, b4);
   if constexpr (AFTER == kUpdate) {
     ld4(a.dinv + node * 4, q4);
@@ -1177,9 +1180,9 @@ __global__ void __launch_bounds__(256) k_ns_nodes(const NsNodeArgs<T> a) {
 #pragma unroll
       for (int f = 0; f < 4; ++f) sum[f] += tl[k][f];
   }
-  const bool bnd = ix == 0 || ix == M - 1 || iy == 0 || iy == M - 1 || iz == 0 || iz == M - 1;
+  if (bnd)  // identity rows
 #pragma unroll
-  for (int f = 0; f < 3; ++f) sum[f] = bnd ? x4[f] : sum[f];  // identity rows
+    for (int f = 0; f < 3; ++f) sum[f] = x4[f];
   if constexpr (AFTER == kStore) {
     st4(a.dst + node * 4, sum);
   } else if constexpr (AFTER == kResidual) {
