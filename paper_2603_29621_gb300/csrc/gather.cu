@@ -67,7 +67,7 @@ __device__ __forceinline__ void gather_one(const GatherArgs<T>& a, const T* buf,
   T x[NU], bb[NU], qq[NU], dd[NU];
 #pragma unroll
   for (int f = 0; f < NU; ++f) {
-    if (AFTER != 3) x[f] = a.src[dof + f];
+    if (AFTER == 1 || (AFTER != 3 && ((m >> f) & 1u))) x[f] = a.src[dof + f];  // the iterate, or identity rows
     if (AFTER == 1 || AFTER == 2) bb[f] = a.b[dof + f];
     if (AFTER == 1) {
       qq[f] = a.dinv[dof + f];
