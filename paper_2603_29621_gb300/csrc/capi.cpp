@@ -100,8 +100,12 @@ int mfns_ctx_set_batching(mfns_ctx* ctx, int enable) {
   return MFNS_OK;
 }
 
+void CtxRef::release(mfns_ctx* c) {
+  if (c && --c->refs == 0) delete c;
+}
+
 int mfns_ctx_destroy(mfns_ctx* ctx) {
-  delete ctx;
+  CtxRef::release(ctx);
   return MFNS_OK;
 }
 

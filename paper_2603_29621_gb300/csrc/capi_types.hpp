@@ -1,5 +1,6 @@
 // Definitions of the opaque C-ABI handles (shared by the C-ABI translation units).
 #pragma once
+#include <atomic>
 #include <memory>
 #include <utility>
 #include <vector>
@@ -22,16 +23,39 @@ struct BatchRound {
 };
 
 struct mfns_ctx {
+  std::atomic<int> refs{1};  // the caller's handle and everything made with the context
   int device = 0;
   mfns::Budget budget;
   bool batching = true;  // mfns_batch_step batches eligible preconditioners
   std::unique_ptr<BatchRound> round;
 };
 
+// A context's use by a mesh, problem or slab, whose buffers are counted against its budget: handles may be
+// destroyed in any order (a garbage collector does so).
+class CtxRef {
+ public:
+  CtxRef() = default;
+  CtxRef(const CtxRef& o) : CtxRef() { *this = o.c_; }
+  CtxRef& operator=(const CtxRef& o) { return *this = o.c_; }
+  CtxRef& operator=(mfns_ctx* c) {
+    if (c) ++c->refs;
+    release(c_);
+    c_ = c;
+    return *this;
+  }
+  ~CtxRef() { release(c_); }
+  operator mfns_ctx*() const { return c_; }
+  mfns_ctx* operator->() const { return c_; }
+  static void release(mfns_ctx* c);
+
+ private:
+  mfns_ctx* c_ = nullptr;
+};
+
 // plan of a batched round over `ps` (cached in the context while the set is unchanged)
 BatchRound* batch_round(mfns_ctx* ctx, const std::vector<mfns::Problem*>& ps);
 struct mfns_mesh {
-  mfns_ctx* ctx = nullptr;
+  CtxRef ctx;
   mfns::Forest forest;
 };
 // Staging of mfns_vmult_host: two device input and output sets of one (operator, precision),
@@ -51,7 +75,7 @@ struct HostIO {
 };
 
 struct mfns_problem {
-  mfns_ctx* ctx = nullptr;
+  CtxRef ctx;  // first: outlives the buffers
   std::unique_ptr<HostIO> hio;  // declared before p: destroyed after it
   std::unique_ptr<mfns::Problem> p;
 };

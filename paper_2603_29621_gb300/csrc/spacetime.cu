@@ -195,7 +195,7 @@ struct Stmg {
 }  // namespace mfns
 
 struct mfns_spacetime {
-  mfns_ctx* ctx = nullptr;
+  CtxRef ctx;  // first: outlives the buffers
   mfns::Budget* bud = nullptr;
   mfns_problem* problem = nullptr;  // Taylor--Hood slabs: not owned, outlives the slab
   std::unique_ptr<mfns::StmgLevel> top;  // P^disc slabs: the slab's own space (FP64)
