@@ -1359,7 +1359,7 @@ BatchVcyclePtr make_batch_vcycle(const std::vector<Problem*>& ps, int prec, cons
 }
 
 // One smoothing sweep of every member of a group: the same steps as smooth_t (without fusion),
-// the operator applications of all members in one multi-problem launch per colour.
+// the operator applications of all members in multi-problem launches.
 template <typename T>
 static void batch_smooth(BatchVcycle& B, int t, BatchGroup& G, bool x_is_zero, cudaStream_t s) {
   const int prec = B.prec;

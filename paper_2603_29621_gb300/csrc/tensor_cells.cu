@@ -6,11 +6,13 @@
 // matrices of the velocity and pressure bases.  Seven 1D contractions replace the twelve of
 // interpolation, derivatives and their transposes.
 //
-// One thread owns one component of one cell: its (k + 1)^3 <= 27 values, the two intermediate fields
-// and the hanging-node interpolation stay in registers, and nothing is exchanged but the sum of the
-// three components' divergence (two shuffles per pressure value).  Degrees 3 and 4: lines, below.  Three adjacent lanes share a cell,
-// ten cells a warp; tables are uniform operands and index lists are stored by slot, so their loads are
-// consecutive over cells.  Bound by instruction issue and the latency of the gather.
+// FP32, degrees 1 and 2: one thread owns one component of one cell: its (k + 1)^3 <= 27 values, the two
+// intermediate fields and the hanging-node interpolation stay in registers, and nothing is exchanged but
+// the sum of the three components' divergence (two shuffles per pressure value).  Three adjacent lanes
+// share a cell, ten cells a warp; tables are uniform operands and index lists are stored by slot, so
+// their loads are consecutive over cells.  Bound by instruction issue and the latency of the gather
+// (Stokes Q2/Q1, 24^3 with two refinements, whole product against the general kernel 70 -> 30 us).
+// FP64 and degrees 3 and 4: lines, below.
 #include <atomic>
 #include <type_traits>
 
@@ -340,10 +342,11 @@ __global__ void __launch_bounds__(128) k_tensor_cells(const __grid_constant__ Tp
   }
 }
 
-// ------------------------------------------------------------------------------- degrees 3 and 4: lines
-// A component's (k + 1)^3 values no longer fit a thread: a thread owns one line of one component, and the
-// fields go through shared memory between the directions, three stages and two barriers (six more in a
-// block with hanging nodes).  FP64 products are bound by the number of operations.
+// ------------------------------------------------------------------------ FP64, degrees 3 and 4: lines
+// A component's (k + 1)^3 values no longer fit a thread, or (FP64) one thread's operations take too long
+// in a row: a thread owns one line of one component, and the fields go through shared memory between the
+// directions, three stages and two barriers (six more in a block with hanging nodes).  FP64 products are
+// bound by the number of operations (Stokes Q3/Q2 24^3 341 -> 249 us).
 template <int N, int NP, int KIND, int TH>
 struct TpLines {
   static constexpr int NL = N * N, NB = NL * N, NBP = NP * NP * NP, COMP = KIND == 2 ? 1 : 3;
