@@ -21,7 +21,8 @@
  *     No C++ exception crosses this boundary.
  *   - Vectors passed as `const void*` / `void*` are DEVICE pointers owned by
  *     the caller (for example the data pointers of torch tensors), laid out as
- *     described in mfns_problem_info and aligned to 16 bytes.  They are read
+ *     described in mfns_problem_info and aligned to 16 bytes (except where a
+ *     call says otherwise).  They are read
  *     and written asynchronously on `stream` (a cudaStream_t, NULL = the
  *     legacy default stream); the caller synchronises.  src and dst must not
  *     alias.  Host pointers are only used where the name says so (`_host`).
@@ -287,7 +288,8 @@ int mfns_kernel_timing(mfns_problem* p, int which, int mode, double* total_ms, i
 /* ---- multigrid ----------------------------------------------------------------------------- */
 /* One smoothing step on level `level`: Chebyshev of the problem's degree (or the Jacobi
  * relaxation) around point Jacobi, starting from x (x_is_zero = 1 skips the first product);
- * b and x have n = level_dofs[level] entries. */
+ * b and x have n = level_dofs[level] entries; any alignment (vectors that the level's kernels could not
+ * read in place are copied through a workspace of the level). */
 int mfns_smooth(mfns_problem* p, int level, int precision, const void* b, void* x, int64_t n, int x_is_zero,
                 void* stream);
 /* Same smoothing step as mfns_smooth, for callers that must not allocate device memory
@@ -306,7 +308,7 @@ int mfns_smooth_noalloc(mfns_problem* p, int level, int precision, const void* b
                         int x_is_zero, void* stream);
 /* Transfers between level `level` (fine) and level+1 (coarse), Eq. 4:
  * fine += P coarse;  coarse = P^T fine.  n_fine = level_dofs[level], n_coarse =
- * level_dofs[level + 1]. */
+ * level_dofs[level + 1].  Vectors of any alignment, as for mfns_smooth. */
 int mfns_prolongate_add(mfns_problem* p, int level, int precision, const void* coarse, int64_t n_coarse,
                         void* fine, int64_t n_fine, void* stream);
 int mfns_restrict(mfns_problem* p, int level, int precision, const void* fine, int64_t n_fine, void* coarse,

@@ -76,6 +76,20 @@ BatchRound* batch_round(mfns_ctx* ctx, const std::vector<Problem*>& ps) {
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The kernels of four-component levels (stabilised operator in 3D) access vectors 16 bytes at a time.
+// mfns_smooth and the transfers take vectors of any alignment: a misaligned one goes through a
+// workspace of its level that the call does not use otherwise.
+static bool staged(const OpLevel& lv, const void* v) { return lv.NU == 4 && !aligned16(v); }
+static const void* stage_in(const OpLevel& lv, int prec, const void* v, const DevBuf& spare, cudaStream_t s) {
+  if (!staged(lv, v)) return v;
+  MFNS_CUDA(cudaMemcpyAsync(spare.get(), v, (size_t)lv.n_dofs * esize(prec), cudaMemcpyDeviceToDevice, s));
+  return spare.get();
+}
+static void* stage_out(const OpLevel& lv, void* v, const DevBuf& spare) { return staged(lv, v) ? spare.get() : v; }
+static void stage_back(const OpLevel& lv, int prec, void* v, const void* at, cudaStream_t s) {
+  if (at != v) MFNS_CUDA(cudaMemcpyAsync(v, at, (size_t)lv.n_dofs * esize(prec), cudaMemcpyDeviceToDevice, s));
+}
+
 extern "C" {
 
 const char* mfns_last_error(void) { return g_err.c_str(); }
@@ -432,7 +446,13 @@ int mfns_smooth(mfns_problem* p, int level, int prec, const void* b, void* x, in
   if (p->p->ls) return fail(MFNS_ERR_UNSUPPORTED, "single-level smoothing is not exposed for local smoothing");
   CHECK_LEN(n, p->p->levels[level]->n_dofs, "b/x");
   MFNS_CUDA(cudaSetDevice(p->ctx->device));
-  smooth(*p->p, level, prec, b, x, x_is_zero != 0, S(stream));
+  const OpLevel& lv = *p->p->levels[level];
+  const Workspace& w = p->p->ws[prec][level];
+  const void* bs = stage_in(lv, prec, b, w.b, S(stream));
+  void* xs = stage_out(lv, x, w.x);
+  if (!x_is_zero) stage_in(lv, prec, x, w.x, S(stream));
+  smooth(*p->p, level, prec, bs, xs, x_is_zero != 0, S(stream));
+  stage_back(lv, prec, x, xs, S(stream));
   API_END
 }
 
@@ -445,7 +465,13 @@ int mfns_prolongate_add(mfns_problem* p, int level, int prec, const void* coarse
   CHECK_LEN(n_coarse, P.levels[level + 1]->n_dofs, "coarse");
   CHECK_LEN(n_fine, P.levels[level]->n_dofs, "fine");
   MFNS_CUDA(cudaSetDevice(p->ctx->device));
-  transfer_prolongate_add(*P.transfers[level], *P.levels[level], *P.levels[level + 1], prec, coarse, fine, S(stream));
+  const OpLevel &f = *P.levels[level], &c = *P.levels[level + 1];
+  const DevBuf& spare = P.ws[prec][level].r;
+  const void* cs = stage_in(c, prec, coarse, P.ws[prec][level + 1].x, S(stream));
+  stage_in(f, prec, fine, spare, S(stream));
+  void* fs = stage_out(f, fine, spare);
+  transfer_prolongate_add(*P.transfers[level], f, c, prec, cs, fs, S(stream));
+  stage_back(f, prec, fine, fs, S(stream));
   API_END
 }
 
@@ -458,7 +484,11 @@ int mfns_restrict(mfns_problem* p, int level, int prec, const void* fine, int64_
   CHECK_LEN(n_fine, P.levels[level]->n_dofs, "fine");
   CHECK_LEN(n_coarse, P.levels[level + 1]->n_dofs, "coarse");
   MFNS_CUDA(cudaSetDevice(p->ctx->device));
-  transfer_restrict(*P.transfers[level], *P.levels[level], *P.levels[level + 1], prec, fine, coarse, S(stream));
+  const OpLevel &f = *P.levels[level], &c = *P.levels[level + 1];
+  const void* fs = stage_in(f, prec, fine, P.ws[prec][level].r, S(stream));
+  void* cs = stage_out(c, coarse, P.ws[prec][level + 1].b);
+  transfer_restrict(*P.transfers[level], f, c, prec, fs, cs, S(stream));
+  stage_back(c, prec, coarse, cs, S(stream));
   API_END
 }
 
@@ -620,6 +650,8 @@ int mfns_batch_vcycle(mfns_problem** ps, int n, int precision, void* const* b, v
     CHECK_LEN(lengths[i], ps[i]->p->levels[0]->n_dofs, "b[i]/x[i]");
     if (!batchable(*ps[i]->p))
       return fail(MFNS_ERR_UNSUPPORTED, "batched V-cycle: one-V-cycle problems on uniform levels only");
+    if (staged(*ps[i]->p->levels[0], x[i]) && ps[i]->p->levels.size() > 1)
+      return fail(MFNS_ERR_ARG, "x[i] must be 16-byte aligned");  // operand of products
     pp.push_back(ps[i]->p.get());
     bb.push_back(b[i]);
     xx.push_back(x[i]);

@@ -86,6 +86,10 @@ extern "C" int mfns_smooth_noalloc(mfns_problem* p, int level, int precision, co
     if (n > kMaxEntries)
       return capi_fail(kErrArg, ("mfns_smooth_noalloc: level has " + std::to_string(n) +
                                  " entries, the fixed scratch holds at most 1048576 per vector").c_str());
+    // x is the operand of products, which read four components at a time
+    if (p->p->levels[level]->NU == 4 && (reinterpret_cast<uintptr_t>(x) & 15u) != 0 &&
+        (!x_is_zero || p->p->smoother_degree > 1))
+      return capi_fail(kErrArg, "x must be 16-byte aligned");
     const int dev = p->ctx->device;
     if (dev < 0 || dev >= kMaxDevices) return capi_fail(kErrArg, "device ordinal out of range");
     MFNS_CUDA(cudaSetDevice(dev));
