@@ -110,12 +110,17 @@ int64_t frozen_point_values_per_cell(int dim, int k) {
   return lanes * q * ((nfq + 3) / 4) * 4;
 }
 
-void op_precompute_frozen(const OpLaunch& L, int prec, cudaStream_t s) {
-  if (L.op != OP_STAB_NS || (!L.fq[prec] && !L.lq[prec])) return;
-  if (prec == 0)
-    dispatch<double>(L, nullptr, nullptr, false, s, 2);
-  else
-    dispatch<float>(L, nullptr, nullptr, false, s, 2);
+// nothing to do: an ordinary launch, which starts when everything before it in the stream is complete
+__global__ void k_frozen_ready() {}
+
+void op_precompute_frozen(const OpLaunch& L, cudaStream_t s) {
+  if (L.op != OP_STAB_NS || (!L.fq[0] && !L.lq[0])) return;
+  dispatch<double>(L, nullptr, nullptr, false, s, 2);
+  dispatch<float>(L, nullptr, nullptr, false, s, 2);
+  // products start early and read the point values, as constant data, before they wait for the launch
+  // before them: that launch must not be the one that writes the values
+  k_frozen_ready<<<1, 1, 0, s>>>();
+  MFNS_CUDA(cudaGetLastError());
 }
 
 void op_residual(const OpLaunch& L, int prec, void* dst, cudaStream_t s) {

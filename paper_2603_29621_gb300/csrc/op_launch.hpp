@@ -76,8 +76,9 @@ int autotune_warps(OpLaunch& L, int prec, void* src, void* dst, int64_t n, cudaS
 
 // Stabilised NS: number of precomputed values per cell (lanes x points x values per point).
 int64_t frozen_point_values_per_cell(int dim, int k);
-// Fill L.fq[prec] (device buffer of n_cells * frozen_point_values_per_cell) or L.lq[prec] from the frozen state.
-void op_precompute_frozen(const OpLaunch& L, int prec, cudaStream_t s);
+// Fill L.fq (device buffers of n_cells * frozen_point_values_per_cell) or L.lq, in both precisions, from the
+// frozen state; complete before whatever follows in the stream starts, programmatic dependents too.
+void op_precompute_frozen(const OpLaunch& L, cudaStream_t s);
 
 // Stabilised NS: dst = F(frozen state), the nonlinear residual on the free rows (dst zeroed by the
 // caller; constrained rows untouched).

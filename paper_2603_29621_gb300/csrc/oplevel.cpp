@@ -208,8 +208,8 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
         // spare slots of the last block hold zeros; the tails that no block writes are not read
         MFNS_CUDA(cudaMemset(lv.fq[prec].get(), 0, ns_fq_bytes(L, prec)));
         L.lq[prec] = lv.fq[prec].get();
-        op_precompute_frozen(L, prec, 0);
       }
+      op_precompute_frozen(L, 0);
       MFNS_CUDA(cudaStreamSynchronize(0));
     } else if (ph.precompute_frozen) {
       // point values of the frozen state (u, grad u, Rbar, tau), computed once by the cell kernel
@@ -217,8 +217,8 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
       for (int prec = 0; prec < 2; ++prec) {
         lv.fq[prec].alloc(bud, (size_t)nc * per_cell * esize(prec));
         L.fq[prec] = lv.fq[prec].get();
-        op_precompute_frozen(L, prec, 0);
       }
+      op_precompute_frozen(L, 0);
       MFNS_CUDA(cudaStreamSynchronize(0));
     }
   }

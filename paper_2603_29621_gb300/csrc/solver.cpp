@@ -1172,11 +1172,7 @@ void set_state_fine(Problem& p, double dt, double alpha, const double* U, const 
     oplevel_distribute(f0, 0, f0.gexp[0].get(), s);
     vcast_d2f(f0.gexp[1].as<float>(), f0.gexp[0].as<double>(), f0.n_main_dofs, s);
   }
-  for (int prec = 0; prec < 2; ++prec) op_precompute_frozen(f0.L, prec, s);
-  // a product's cell kernel starts early and reads the point values as constant data: keep a full
-  // completion between the pass that wrote them and the next product of the stream
-  void* between = f0.rows[0].get() ? f0.rows[0].get() : f0.gather ? f0.gather->buf[0].get() : nullptr;
-  if (between) MFNS_CUDA(cudaMemsetAsync(between, 0, 16, s));
+  op_precompute_frozen(f0.L, s);
 }
 
 void refresh_preconditioner(Problem& p, cudaStream_t s) {
@@ -1195,7 +1191,7 @@ void refresh_preconditioner(Problem& p, cudaStream_t s) {
       oplevel_distribute(c, 0, c.gexp[0].get(), s);
       vcast_d2f(c.gexp[1].as<float>(), c.gexp[0].as<double>(), c.n_main_dofs, s);
     }
-    for (int prec = 0; prec < 2; ++prec) op_precompute_frozen(c.L, prec, s);
+    op_precompute_frozen(c.L, s);
   }
   for (auto& lvp : p.levels) level_dinv(p, *lvp, s, true);
   setup_coarse(p, s);  // synchronises
