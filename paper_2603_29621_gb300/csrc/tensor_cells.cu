@@ -13,8 +13,11 @@
 // their loads are consecutive over cells.  Bound by instruction issue and the latency of the gather
 // (Stokes Q2/Q1, 24^3 with two refinements, whole product against the general kernel 70 -> 30 us).
 // FP64 and degrees 3 and 4: lines, below.
+#include <array>
 #include <atomic>
+#include <cmath>
 #include <type_traits>
+#include <vector>
 
 #include "common.hpp"
 #include "op_kernel.cuh"
@@ -649,47 +652,92 @@ bool tensor_cells(const OpLaunch& L) {
                         (L.op == OP_STOKES && L.k >= 2 && L.k <= 4));
 }
 
+// 1D integrals on the reference interval of the bases of degree k (a) and k - 1 (p) on their
+// Gauss--Lobatto nodes, exact in extended precision: polynomials in t = 2 x - 1.  Every product of three
+// tables then carries their roundings alone; formed by a Gauss sum in FP64, the tables were off by up
+// to 9e-15 and the products' error by 1.1 to 1.8 times that of quadrature (Q2 vector Laplacian FP64,
+// 5^3 cells: quadrature 3.7e-16, Gauss-sum tables 6.6e-16, these 1.3e-16).
+struct Integrals {
+  long double m[5][5], k[5][5], mr[5][5], dr[5][5];  // a a, a' a', a p, a' p
+};
+using Poly = std::vector<long double>;
+static std::vector<Poly> lobatto_basis(int k) {
+  const long double c = k == 3 ? 1 / sqrtl(5.0L) : sqrtl(3.0L / 7.0L);
+  const std::vector<long double> t = k == 0   ? std::vector<long double>{0}
+                                     : k == 1 ? std::vector<long double>{-1, 1}
+                                     : k == 2 ? std::vector<long double>{-1, 0, 1}
+                                     : k == 3 ? std::vector<long double>{-1, -c, c, 1}
+                                              : std::vector<long double>{-1, -c, 0, c, 1};
+  std::vector<Poly> out;
+  for (int a = 0; a <= k; ++a) {
+    Poly p{1};
+    for (int m = 0; m <= k; ++m) {
+      if (m == a) continue;
+      p.push_back(0);
+      for (size_t i = p.size(); i-- > 0;) p[i] = ((i ? p[i - 1] : 0) - t[m] * p[i]) / (t[a] - t[m]);
+    }
+    out.push_back(p);
+  }
+  return out;
+}
+static const Integrals& integrals(int k) {
+  static const std::array<Integrals, 5> all = [] {
+    std::array<Integrals, 5> r{};
+    auto derivative = [](const Poly& p) {  // with respect to x
+      Poly d;
+      for (size_t i = 1; i < p.size(); ++i) d.push_back(2 * (long double)i * p[i]);
+      return d;
+    };
+    auto integral = [](const Poly& p, const Poly& q) {
+      long double v = 0;
+      for (size_t i = 0; i < p.size(); ++i)
+        for (size_t j = i % 2; j < q.size(); j += 2) v += p[i] * q[j] / (long double)(i + j + 1);
+      return v;
+    };
+    for (int k = 1; k <= 4; ++k) {
+      const std::vector<Poly> a = lobatto_basis(k), p = lobatto_basis(k - 1);
+      for (int i = 0; i <= k; ++i) {
+        for (int j = 0; j <= k; ++j) {
+          r[k].m[i][j] = integral(a[i], a[j]);
+          r[k].k[i][j] = integral(derivative(a[i]), derivative(a[j]));
+        }
+        for (int j = 0; j < k; ++j) {
+          r[k].mr[i][j] = integral(a[i], p[j]);
+          r[k].dr[i][j] = integral(derivative(a[i]), p[j]);
+        }
+      }
+    }
+    return r;
+  }();
+  return all[k];
+}
+
 template <int N, int NP, int KIND, typename T>
 static void launch(const OpLaunch& L, const NodeGather& g, int prec, const void* src, cudaStream_t s) {
   TpArgs<T, N, NP> a{};
-  // 1D integrals on the reference interval by the level's Gauss rule (exact)
-  auto integral = [&](auto f) {
-    double v = 0.0;
-    for (int q = 0; q < L.Q; ++q) v += L.W[q] * f(q);
-    return v;
-  };
-  auto S = [&](int q, int i) { return L.S[q * N + i]; };
-  auto dS = [&](int q, int i) {
-    double v = 0.0;
-    for (int r = 0; r < L.Q; ++r) v += L.D[q * L.Q + r] * L.S[r * N + i];
-    return v;
-  };
-  double m1[N][N], k1[N][N];
-  for (int i = 0; i < N; ++i)
-    for (int j = 0; j < N; ++j) {
-      m1[i][j] = integral([&](int q) { return S(q, i) * S(q, j); });
-      k1[i][j] = integral([&](int q) { return dS(q, i) * dS(q, j); });
-      for (int hf = 0; hf < 2; ++hf) a.tab.P[hf][i][j] = (T)L.P[(hf * N + i) * N + j];
-    }
-  auto fold = [](const double (&x)[N][N], auto& t) {
+  const Integrals& I = integrals(N - 1);
+  for (int hf = 0; hf < 2; ++hf)
+    for (int i = 0; i < N; ++i)
+      for (int j = 0; j < N; ++j) a.tab.P[hf][i][j] = (T)L.P[(hf * N + i) * N + j];
+  auto fold = [](const long double (&x)[5][5], auto& t) {
     constexpr int H = N / 2;
     for (int i = 0; i < H; ++i) {
       for (int j = 0; j < H; ++j) {
-        t.e[i][j] = (T)(0.5 * (x[i][j] + x[i][N - 1 - j]));
-        t.o[i][j] = (T)(0.5 * (x[i][j] - x[i][N - 1 - j]));
+        t.e[i][j] = (T)(0.5L * (x[i][j] + x[i][N - 1 - j]));
+        t.o[i][j] = (T)(0.5L * (x[i][j] - x[i][N - 1 - j]));
       }
       t.col[i] = (T)x[i][H];
       t.row[i] = (T)x[H][i];
     }
     t.mid = (T)x[H][H];
   };
-  fold(m1, a.tab.M);
-  fold(k1, a.tab.K);
+  fold(I.m, a.tab.M);
+  fold(I.k, a.tab.K);
   if (KIND == 1)
     for (int i = 0; i < N; ++i)
       for (int m = 0; m < NP; ++m) {
-        a.tab.Mr[i][m] = (T)integral([&](int q) { return S(q, i) * L.Sp[q * NP + m]; });
-        a.tab.Dr[i][m] = (T)integral([&](int q) { return dS(q, i) * L.Sp[q * NP + m]; });
+        a.tab.Mr[i][m] = (T)I.mr[i][m];
+        a.tab.Dr[i][m] = (T)I.dr[i][m];
       }
   if (KIND == 1)
     for (int hf = 0; hf < 2; ++hf)
