@@ -819,14 +819,23 @@ __global__ void __launch_bounds__(128) k_ns_items(const __grid_constant__ NsArgs
 // FP32 threads own a whole z-plane of points of a cell (Q x Q points, four fields in registers): the x
 // and y contractions need no exchange at all, the z contractions one pass of 16-byte words through
 // shared memory each way.  Bound by the DRAM stream of the point values; the line kernel above, with
-// a thread per line, is bound by shared-memory bandwidth here (Q2 64^3: 125 us against 103 us for the
+// a thread per line, is bound by shared-memory bandwidth here (Q2 64^3: 125 us against 95 us for the
 // cells alone), but its shorter threads are faster on levels without full blocks (Q2 8^3 and below:
 // 5.2 us against 6.8 us).
+//
+// For Q = 4 the loop over the rows of points stays a loop (ROLL): unrolled, the kernel is 97 KB of
+// instructions, which a pass behind other kernels waits for (Q3 31^3, product: first pass on new vectors
+// 95 us, repeated 58 us; rolled, 55 KB: 76 and 51 us; the colour launches that both replace 84 and 61 us).
+// The loop turns the rows of the registers, so that the current one keeps its place (Q = 3 is faster
+// unrolled: 64^3 130 us against 143 us), and asks for no prefetch of the block's point values: its loads wait
+// behind it (8 warps a SM; rolled with the prefetch 79 and 54 us).
 template <int K>
 struct NsPlane {
   static constexpr int Q = K + 1, NL = Q * Q, THREADS = 32 * Q;
   static constexpr int MINB = Q == 2 ? 8 : Q == 3 ? 5 : 2;
+  static constexpr bool ROLL = Q == 4;
   static constexpr int RING = Q == 3 ? 2 : 4;  // points of a thread's plane on their way (shared memory allows)
+  static_assert(!ROLL || RING == Q, "rolled rows: the slot of a point is its place in the row");
   static constexpr size_t BUF = (size_t)NL * Q * 32 * 16;
   static constexpr size_t SMEM = 2 * BUF + (size_t)RING * 4 * THREADS * 16;
 };
@@ -848,7 +857,7 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
   T* Z = E + NL * Q * 32 * 4;
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const T* fqb = P.fq + ns_fq_at<T, Q>(blk, 0, 0, 0, 0, 0, C);
-  if (threadIdx.x == 0) {  // the block's point values (constant data) towards the L2
+  if (!NsPlane<K>::ROLL && threadIdx.x == 0) {  // the block's point values (constant data) towards the L2
     const unsigned bytes = (unsigned)(NL * Q * 64) * (unsigned)C;
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(fqb), "r"(bytes) : "memory");
   }
@@ -858,17 +867,17 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
   const float4* fp = reinterpret_cast<const float4*>(fqb) + (int64_t)l * 4 * C + fl;
   const float4* ring = reinterpret_cast<const float4*>(ns_smem + 2 * NsPlane<K>::BUF) + threadIdx.x;
   const unsigned ring_s = (unsigned)__cvta_generic_to_shared(ring);
-  auto fetch = [&](int pt) {  // a group per point, empty past the last one
+  auto fetch = [&](int pt, int slot) {  // a group per point, empty past the last one
     if (pt < NL)
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(ring_s + (unsigned)((pt % RING * 4 + q) * NT * 16)),
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(ring_s + (unsigned)((slot * 4 + q) * NT * 16)),
                      "l"(fp + ((int64_t)pt * Q * 4 + q) * C)
                      : "memory");
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
 #pragma unroll
-  for (int pt = 0; pt < RING; ++pt) fetch(pt);
+  for (int pt = 0; pt < RING; ++pt) fetch(pt, pt);
   const uint32_t t = (uint32_t)blk * (uint32_t)C + (uint32_t)lane;
   const bool valid = lane < C && t < P.cells;
   const uint32_t tt = t < P.cells ? t : P.cells - 1;
@@ -948,29 +957,35 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
     for (int j = 0; j < Q; ++j)
 #pragma unroll
       for (int i = 0; i < Q; ++i) acc[f][j][i] = T(0);
-#pragma unroll
+  constexpr bool ROLL = NsPlane<K>::ROLL;
+  constexpr int UNROLL = ROLL ? 1 : Q;
+#pragma unroll UNROLL
   for (int j = 0; j < Q; ++j) {
+    // register row r of val and acc: row of points at(r); the current one is r = j0
+    const int j0 = ROLL ? 0 : j;
+    auto at = [&](int r) { return ROLL ? (j + r) % Q : r; };
     T dx[4][Q], xx[4][Q], cxr[4][Q];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.hD, tab.D2, val[f][j], dx[f], xx[f]);
-    line_deriv<Q, false>(tab.D, tab.hD, tab.D2, val[3][j], dx[3], xx[3]);
+    for (int f = 0; f < 3; ++f) line_deriv<Q, true>(tab.D, tab.hD, tab.D2, val[f][j0], dx[f], xx[f]);
+    line_deriv<Q, false>(tab.D, tab.hD, tab.D2, val[3][j0], dx[3], xx[3]);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       T F[4][4];
+      const int slot = ROLL ? i : (i + Q * j) % RING;
       asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 1) : "memory");
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float4 v4 = ring[((i + Q * j) % RING * 4 + q) * NT];
+        const float4 v4 = ring[(slot * 4 + q) * NT];
         F[q][0] = v4.x; F[q][1] = v4.y; F[q][2] = v4.z; F[q][3] = v4.w;
       }
       T gx[4], gy[4], gz[4], v[4], lap[3], c0[4], cxp[4], cyp[4], czp[4];
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
-        v[f] = val[f][j][i];
+        v[f] = val[f][j0][i];
         gx[f] = dx[f][i];
-        T s = mul_rn(tab.D[j][0], val[f][0][i]);
+        T s = mul_rn(tab.D[j][at(0)], val[f][0][i]);
 #pragma unroll
-        for (int a = 1; a < Q; ++a) s = fma(tab.D[j][a], val[f][a][i], s);
+        for (int a = 1; a < Q; ++a) s = fma(tab.D[j][at(a)], val[f][a][i], s);
         gy[f] = s;
       }
 #pragma unroll
@@ -978,7 +993,7 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
         lap[f] = Q > 2 ? xx[f][i] : T(0);
         if (Q > 2)
 #pragma unroll
-          for (int a = 0; a < Q; ++a) lap[f] = fma(tab.D2[j][a], val[f][a][i], lap[f]);
+          for (int a = 0; a < Q; ++a) lap[f] = fma(tab.D2[j][at(a)], val[f][a][i], lap[f]);
       }
 #pragma unroll
       for (int c = 0; c < Q; ++c) {
@@ -992,19 +1007,34 @@ k_ns_planes(const __grid_constant__ NsArgs<float, K + 1> args) {
           for (int f = 0; f < 3; ++f) lap[f] = fma(d2, e[f], lap[f]);
       }
       ns_point<T>(v, gx, gy, gz, lap, F, P, c0, cxp, cyp, czp);
-      fetch(i + Q * j + RING);  // into the slots just read
+      fetch(i + Q * j + RING, slot);  // into the slots just read
       ns_st(Z, NL * l + i + Q * j, lane, 32, czp[0], czp[1], czp[2], czp[3]);
       const T dl = tab.Dw[l][l];
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         cxr[f][i] = cxp[f];
-        acc[f][j][i] += fma(dl, czp[f], c0[f]);
+        acc[f][j0][i] += fma(dl, czp[f], c0[f]);
 #pragma unroll
-        for (int a = 0; a < Q; ++a) acc[f][a][i] = fma(tab.Dw[a][j], cyp[f], acc[f][a][i]);
+        for (int a = 0; a < Q; ++a) acc[f][a][i] = fma(tab.Dw[at(a)][j], cyp[f], acc[f][a][i]);
       }
     }
 #pragma unroll
-    for (int f = 0; f < 4; ++f) line_dwt<Q, true>(tab.Dw, tab.hDw, cxr[f], acc[f][j]);
+    for (int f = 0; f < 4; ++f) line_dwt<Q, true>(tab.Dw, tab.hDw, cxr[f], acc[f][j0]);
+    if constexpr (ROLL) {
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          const T v0 = val[f][0][i], a0 = acc[f][0][i];
+#pragma unroll
+          for (int r = 0; r + 1 < Q; ++r) {
+            val[f][r][i] = val[f][r + 1][i];
+            acc[f][r][i] = acc[f][r + 1][i];
+          }
+          val[f][Q - 1][i] = v0;
+          acc[f][Q - 1][i] = a0;
+        }
+    }
   }
   __syncthreads();
   // ---- test side: z derivatives of the other planes, then the transposed values y, x and z
