@@ -878,8 +878,8 @@ def run_ours(args, world, rank, local):
     clocks.wait_ready()
     clocks.mark()
     ms32 = timed(lambda: prob.vmult(src32, dst32), args.steps, args.warmup, nvtx="timed_vmult_fp32")
-    # ---- the cell kernel's launches, each bracketed by CUDA events on the launching stream (the
-    # events serialise the launches): the per-launch roofline figure
+    # ---- the product's launches, each bracketed by CUDA events on the launching stream (the events
+    # serialise them): the per-launch roofline figure
     prob.kernel_timing(1)
     timed(lambda: prob.vmult(src32, dst32), args.steps, args.warmup)
     kms, klaunch = prob.kernel_timing(2)
@@ -952,19 +952,6 @@ def run_ours(args, world, rank, local):
         guarded("chebyshev3_fp32", cheb)
         guarded("vcycle_fp32", vcyc)
 
-        def fused():
-            pf = api.Problem(ctx, m, kind=L.STAB_NS, degree=2, nu=1e-2, dt=1e-2, smoother=1, smoother_degree=3,
-                             mg_precision=L.FP32, fused_smoother=1)
-            try:
-                for lvl in range(prob.info.n_levels - 1):
-                    pf.set_lambda_max(lvl, prob.info.lambda_max[lvl])
-                return {"ms_per_sweep": timed(lambda: pf.smooth(0, b32, xs, x_is_zero=False),
-                                              max(3, args.steps // 2), 3, nvtx="timed_cheb_fused"),
-                        "vcycle_ms": timed(lambda: pf.vcycle(b32, xs), steps_s, 3)}
-            finally:
-                pf.close()
-
-        guarded("fused_smoother_fp32", fused)
     prob.close()
     m.close()
     ctx.close()
@@ -984,11 +971,13 @@ def run_ours(args, world, rank, local):
         pass
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     # algorithmic bytes of one apply: src and dst (4 fields each) and the frozen state (u, p: 4
-    # fields) once per node, FP32 -- 12 x 2,146,689 x 4 B = 103.0 MB at 64^3; the cell launch
-    # processes all cells and is charged all of it
+    # fields) once per node, FP32 -- 12 x 2,146,689 x 4 B = 103.0 MB at 64^3, against the time of
+    # both launches of the product (the cells read src, the node pass writes dst)
     alg_bytes = 12 * nodes * 4
     bytes_launch = alg_bytes * cells_per_launch / ncell
     achieved = bytes_launch / (avg_launch_ms * 1e-3) / 1e9
+    rows = n * n * 9 * (2 * n + 1) * 16   # x-rows of node values per cell row and line, 4 fields
+    moved = 8 * nodes * 4 + ncell * FQ_BYTES_PER_CELL_F32 + 2 * rows
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms32, "higher_is_better": True, "scaling": "weak",
@@ -996,7 +985,7 @@ def run_ours(args, world, rank, local):
         "config": headline_config(n, world),
         "clocks": clk,
         # per step: the cell launch and the node pass
-        "gpu_launches": (launches_per_step + 1) * args.steps,
+        "gpu_launches": launches_per_step * args.steps,
         "e2e": {"value": whole_job_rate(ndof, world, ms_e2e), "unit": UNIT, "h2d_bytes_per_step": ndof * 4,
                 "d2h_bytes_per_step": ndof * 4, "ms_per_step": ms_e2e,
                 "how": "C ABI with HOST buffers: one mfns_vmult_host call for all timed steps (pinned "
@@ -1008,12 +997,13 @@ def run_ours(args, world, rank, local):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                      "frac": achieved / hbm_peak, "traffic": traffic,
                      "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy, burst), of measured",
-                     "kernel": "k_ns_planes<2> (the cell launch of a product)",
+                     "kernel": "k_ns_planes<2> and k_ns_nodes<float, 2> (the two launches of a product)",
                      "alg_bytes_per_apply": alg_bytes, "alg_bytes_per_launch": bytes_launch,
                      "alg_bytes_rule": "12 fields (src 4, dst 4, frozen u,p 4) x nodes x 4 B",
                      "cells_per_launch": cells_per_launch, "avg_launch_ms": avg_launch_ms,
-                     "avg_launch_note": "cell launches timed by themselves (events serialise them); the "
-                                        "headline apply adds the node pass, which overlaps their tail",
+                     "avg_launch_note": "mean of the two launches, timed by themselves (events serialise them; "
+                                        "in the headline apply the node pass starts while the cells drain); "
+                                        "bytes and cells per launch are half the product's",
                      "launches_per_apply": launches_per_step,
                      "whole_apply": {"achieved_gbs": alg_bytes / (ms32 * 1e-3) / 1e9,
                                      "frac": alg_bytes / (ms32 * 1e-3) / 1e9 / hbm_peak},
@@ -1022,13 +1012,11 @@ def run_ours(args, world, rank, local):
                              "peak_rule": "152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz"},
                      "ridge_flop_per_byte": peak_alu * 1e12 / (hbm_peak * 1e9),
                      "intensity_flop_per_byte": FLOP_PER_CELL * ncell / alg_bytes,
-                     "with_point_data": {"note": "bytes the product moves by design: src, dst and the "
-                                                 "precomputed point values (1,728 B per cell)",
-                                         "bytes_per_launch": (8 * nodes * 4 * cells_per_launch / ncell
-                                                              + cells_per_launch * FQ_BYTES_PER_CELL_F32),
-                                         "achieved_gbs": (8 * nodes * 4 * cells_per_launch / ncell
-                                                          + cells_per_launch * FQ_BYTES_PER_CELL_F32)
-                                         / (avg_launch_ms * 1e-3) / 1e9}},
+                     "with_point_data": {"note": "bytes the product moves by design: src, dst, the precomputed "
+                                                 "point values (1,728 B per cell), and the rows between its "
+                                                 "launches (written and read, mostly in the L2)",
+                                         "bytes_per_apply": moved, "rows_bytes": rows,
+                                         "achieved_gbs": moved / (launches_per_step * avg_launch_ms * 1e-3) / 1e9}},
     }
     line.update(extra)
     if world == 1 and not args.no_cpu_baseline:

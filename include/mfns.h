@@ -128,11 +128,12 @@ typedef struct {
   int recompute_frozen; /* STAB_NS: 1 = interpolate the frozen state inside every apply; 0 (default) =
                            store its point values (u, grad u, Rbar, tau) once per level (more HBM,
                            fewer shared-memory contractions per apply) */
-  int fused_smoother;   /* 1: on uniform levels the Chebyshev / Jacobi update and the V-cycle residual
-                           are applied by the cell kernel to each node in the colour that completes
-                           its product (no separate vector pass); 0 (default): the product is
-                           written out and a streaming kernel applies the update (faster on GB300:
-                           the cell kernel is latency-bound) */
+  int fused_smoother;   /* levels whose product ends in a node pass apply the Chebyshev / Jacobi update
+                           and the V-cycle residual there, whatever the value.  On uniform levels whose
+                           product runs colour by colour, 1: the cell kernel applies them to each
+                           node in the colour that completes its product; 0 (default): the product
+                           is written out and a streaming kernel applies them (faster on GB300).
+                           1 also keeps the problem's preconditioner out of batched rounds. */
   int hierarchy;        /* multigrid levels on a locally refined mesh (Section 2): 0 (default) global
                            coarsening -- every level covers the whole domain, hanging nodes resolved
                            on each; 1 local smoothing (MFNS_STOKES, MFNS_STOKES_A and
@@ -252,8 +253,9 @@ int mfns_problem_destroy(mfns_problem* p);
 /* ---- operators ----------------------------------------------------------------------------- */
 /* dst = A src (matrix-free, Section 1 / Eq. 4 per cell); constrained rows dst_i = src_i.
  * n: entries of src and of dst (n_dofs for MFNS_OP_SYSTEM, n_dofs - n_velocity_dofs for
- * MFNS_OP_PMASS, level_dofs[which] for a level).  On a uniform mesh the colour launches after
- * the first start while their predecessor drains (programmatic dependent launches). */
+ * MFNS_OP_PMASS, level_dofs[which] for a level).  Two launches, the cells and a pass over the nodes, or one
+ * launch per colour; each but the first starts while its predecessor drains (programmatic dependent
+ * launches). */
 int mfns_vmult(mfns_problem* p, int which, int precision, const void* src, void* dst, int64_t n,
                void* stream);
 /* dst_host[i] = A src_host[i], i < count, for vectors in HOST memory (a list of requests to the same
@@ -272,8 +274,8 @@ int mfns_vmult(mfns_problem* p, int which, int precision, const void* src, void*
  * budget). */
 int mfns_vmult_host(mfns_problem* p, int which, int precision, const void* const* src_host,
                     void* const* dst_host, int count, int64_t n, void* stream);
-/* diag = diag(A) (exact, per-cell unit-vector evaluation; 1 on constrained rows); n as in
- * mfns_vmult. */
+/* diag = diag(A) (exact: from the stored point values on uniform 3D stabilised levels, by per-cell
+ * unit vectors elsewhere; 1 on constrained rows); n as in mfns_vmult. */
 int mfns_diagonal(mfns_problem* p, int which, int precision, void* diag, int64_t n, void* stream);
 /* Hanging entries of x from their masters (x_h = sum_j w_hj x_j), Dirichlet entries kept; n as in
  * mfns_vmult. */
@@ -282,7 +284,9 @@ int mfns_apply_constraints(mfns_problem* p, int which, int precision, void* x, i
 /* Per-kernel timing of the operator-kernel launches of `which` with CUDA events recorded on
  * the launching stream: mode 1 = reset and enable, 0 = disable, 2 = read (synchronises on the
  * recorded events; writes the summed kernel time in ms and the number of timed launches,
- * then resets).  The timed launches are the colour launches of the cell kernel only. */
+ * then resets).  The timed launches are those that make up a product: the cell launch and the node
+ * pass (with the smoother update or the residual that it applies), or the colour launches of the
+ * cell kernel where the level has those; the events keep them from overlapping. */
 int mfns_kernel_timing(mfns_problem* p, int which, int mode, double* total_ms, int64_t* launches);
 
 /* ---- multigrid ----------------------------------------------------------------------------- */

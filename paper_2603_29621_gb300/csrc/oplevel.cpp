@@ -368,19 +368,22 @@ void ensure_gather(OpLevel& lv, int prec, Budget* bud) {
   if (!G.buf[prec].get()) G.buf[prec].alloc(bud, (size_t)(G.main_values() + G.slots_p) * esize(prec));
 }
 
-// a product whose node pass applies what follows it
+// a product whose node pass applies what follows it (timed: both launches; the cell launch records itself)
 static void node_product(const OpLevel& lv, int prec, const NsAfterArgs& a, cudaStream_t s) {
-  if (lv.L.lq[prec]) {
+  const NodeGather* G = lv.L.lq[prec] ? nullptr : lv.gather.get();
+  if (!G)
     ns_cells(lv.L, prec, a.src, lv.rows[prec].get(), s);
-    ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
-    return;
-  }
-  const NodeGather& G = *lv.gather;
-  if (G.tensor)
-    tensor_product(lv.L, G, prec, a.src, s);
+  else if (G->tensor)
+    tensor_product(lv.L, *G, prec, a.src, s);
   else
-    op_apply_deferred(lv.L, prec, a.src, G.buf[prec].get(), G.main_values(), s);
-  gather_nodes(G, prec, a, s);
+    op_apply_deferred(lv.L, prec, a.src, G->buf[prec].get(), G->main_values(), s);
+  const bool timed = lv.L.timer && lv.L.timer->enabled;
+  if (timed) lv.L.timer->record_pair_begin(s);
+  if (!G)
+    ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
+  else
+    gather_nodes(*G, prec, a, s);
+  if (timed) lv.L.timer->record_pair_end(s);
 }
 
 void oplevel_vmult(const OpLevel& lv, int prec, const void* src, void* dst, cudaStream_t s) {
