@@ -37,7 +37,9 @@
  *   - The library owns meshes, hierarchies, diagonals, frozen states and
  *     workspaces; they are allocated against the context's HBM budget at
  *     create time (MFNS_ERR_BUDGET when it would be exceeded), so vmult,
- *     smooth, vcycle and solve allocate nothing.
+ *     smooth, vcycle and solve allocate nothing.  A problem that fits the
+ *     budget only without the buffer and tables of two-launch products
+ *     (2 to 16 % of it) is created without them; its products are slower.
  *   - One problem is used by one stream at a time (not thread-safe per
  *     problem); distinct problems may run concurrently on distinct streams.
  *

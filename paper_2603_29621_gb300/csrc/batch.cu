@@ -45,7 +45,7 @@ static void fill_ns(MultiOp& m, Budget* bud) {
       const int64_t nb = ns_blocks(lv.L, m.prec);
       if (pid.size() + (size_t)nb >= (size_t)1 << 31)
         throw Error(kErrUnsupported, "multi-problem launch: too many blocks");
-      ns_descriptor(lv.L, m.prec, m.src[i], lv.rows[m.prec].get(), (int32_t)(pid.size() - pid_at[kind]), desc);
+      ns_descriptor(lv.L, m.prec, m.src[i], lv.scratch->get(), (int32_t)(pid.size() - pid_at[kind]), desc);
       pid.insert(pid.end(), (size_t)nb, members++);
       m.ns[kind].cmax = std::max(m.ns[kind].cmax, lv.L.lc[m.prec]);
     }
@@ -152,7 +152,7 @@ void multi_vmult(const MultiOp& m, cudaStream_t s) {
       NsAfterArgs a;
       a.dst = m.dst[i];
       a.src = m.src[i];
-      ns_nodes(m.lv[i]->L, m.prec, a, m.lv[i]->rows[m.prec].get(), s);
+      ns_nodes(m.lv[i]->L, m.prec, a, m.lv[i]->scratch->get(), s);
     }
     return;
   }

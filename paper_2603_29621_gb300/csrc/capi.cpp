@@ -182,10 +182,14 @@ int mfns_problem_create(mfns_ctx* ctx, const mfns_mesh* mesh, const mfns_problem
   if (desc->hierarchy != 0 && desc->hierarchy != 1) return fail(MFNS_ERR_ARG, "hierarchy must be 0 or 1");
   if (desc->hierarchy == 1 && desc->kind == MFNS_PMASS)
     return fail(MFNS_ERR_UNSUPPORTED, "local smoothing is built for MFNS_STOKES, MFNS_STOKES_A and MFNS_STAB_NS");
-  std::unique_ptr<Problem> p = build_problem(mesh->forest, desc->kind, k, ph, desc->mg_order,
-                                             desc->coarse_stop_n > 0 ? desc->coarse_stop_n : 2, &ctx->budget,
-                                             desc->hierarchy);
-  return finish_problem(ctx, desc, std::move(p), used0, out);
+  int status = MFNS_OK;
+  build_within_budget(&ctx->budget, [&](const ScratchPtr& scratch) {
+    std::unique_ptr<Problem> p = build_problem(mesh->forest, desc->kind, k, ph, desc->mg_order,
+                                               desc->coarse_stop_n > 0 ? desc->coarse_stop_n : 2, &ctx->budget,
+                                               scratch, desc->hierarchy);
+    status = finish_problem(ctx, desc, std::move(p), used0, out);
+  });
+  return status;
   API_END
 }
 
@@ -239,10 +243,14 @@ int mfns_problem_create_hp(mfns_ctx* ctx, const mfns_mesh* mesh, const mfns_prob
   ph.nu = desc->nu;
   ph.div_sign = -1.0;
   const size_t used0 = ctx->budget.used;
-  std::unique_ptr<Problem> p = build_problem_hp(mesh->forest, degree, ph,
-                                                desc->coarse_stop_n > 0 ? desc->coarse_stop_n : 2, &ctx->budget,
-                                                desc->kind == MFNS_STOKES ? 0 : 1);
-  return finish_problem(ctx, desc, std::move(p), used0, out);
+  int status = MFNS_OK;
+  build_within_budget(&ctx->budget, [&](const ScratchPtr& scratch) {
+    std::unique_ptr<Problem> p = build_problem_hp(mesh->forest, degree, ph,
+                                                  desc->coarse_stop_n > 0 ? desc->coarse_stop_n : 2, &ctx->budget,
+                                                  scratch, desc->kind == MFNS_STOKES ? 0 : 1);
+    status = finish_problem(ctx, desc, std::move(p), used0, out);
+  });
+  return status;
   API_END
 }
 

@@ -33,6 +33,12 @@ struct Error : std::runtime_error {
                                                 " " #expr ": " + cudaGetErrorString(e_));                 \
   } while (0)
 
+// over: bytes by which the allocation would have exceeded the budget
+struct BudgetError : Error {
+  size_t over;
+  explicit BudgetError(size_t o) : Error(kErrBudget, "HBM budget exceeded"), over(o) {}
+};
+
 // Per-context HBM accounting: every library allocation is charged against the budget
 // (thread-safe: problems of one context may be created and destroyed from several threads).
 struct Budget {
@@ -40,7 +46,7 @@ struct Budget {
   std::mutex mu;
   void charge(size_t b) {
     std::lock_guard<std::mutex> lock(mu);
-    if (limit && used + b > limit) throw Error(kErrBudget, "HBM budget exceeded");
+    if (limit && used + b > limit) throw BudgetError(used + b - limit);
     used += b;
     if (used > peak) peak = used;
   }

@@ -144,7 +144,7 @@ static void launch(const NodeGather& g, int prec, const NsAfterArgs& f, cudaStre
   a.b = static_cast<const T*>(f.b);
   a.dinv = static_cast<const T*>(f.dinv);
   a.d = static_cast<T*>(f.d);
-  a.buf = g.buf[prec].as<T>();
+  a.buf = static_cast<const T*>(g.scratch->get());
   a.buf_p = a.buf + g.main_values();
   a.ptr = g.ptr.as<int32_t>();
   a.idx = g.idx.as<int32_t>();

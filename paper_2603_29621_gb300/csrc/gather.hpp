@@ -3,13 +3,51 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <memory>
 #include <vector>
 
 #include "common.hpp"
 #include "ns_lines.hpp"
 
 namespace mfns {
+
+// What lies between the two launches of a product: one buffer for all levels and both precisions of a problem,
+// whose products run one at a time.  Levels without one (null) run colour by colour, and so does a
+// problem that fits its context's budget only then.
+struct ProductScratch {
+  Budget* bud = nullptr;
+  size_t need = 0;    // largest request
+  size_t tables = 0;  // bytes of the levels' tables and layouts that only products through this buffer use
+  explicit ProductScratch(Budget* b) : bud(b) {}
+  void reserve(size_t bytes) {  // while levels are laid out (the contents are dropped)
+    need = std::max(need, bytes);
+    if (buf_.bytes() < need) buf_.alloc(bud, need);
+  }
+  void* get() const { return buf_.get(); }
+
+ private:
+  DevBuf buf_;
+};
+using ScratchPtr = std::shared_ptr<ProductScratch>;
+
+// build(scratch), and build(null) if the budget or the device's memory does not hold the first by no more
+// than what the scratch and its tables take
+template <typename F>
+void build_within_budget(Budget* bud, F build) {
+  ScratchPtr scratch = std::make_shared<ProductScratch>(bud);
+  try {
+    return build(scratch);
+  } catch (const BudgetError& e) {
+    if (e.over > scratch->need + scratch->tables) throw;
+  } catch (const Error& e) {
+    if (e.code != kErrOom || !scratch->need) throw;
+    (void)cudaGetLastError();
+  }
+  scratch.reset();
+  build(nullptr);
+}
 
 // Contributions of a level's nodes: entries e of node g (ptr[g] <= e < ptr[g + 1]) are the places idx[e]
 // in the buffer, ascending.  Place of (cell, slot): position * slots + slot with cells in colour order,
@@ -26,10 +64,10 @@ struct NodeGather {
   DevBuf mask;          // per node (main, then pressure): bit f set where entry f is an identity row
   int64_t n_main = 0, n_p = 0, slots = 0, slots_p = 0;  // nodes; contributions of all cells
   int nu = 1;
-  DevBuf buf[2];        // the contributions per precision: main, then pressure
+  ScratchPtr scratch;   // holds the contributions: main, then pressure
   size_t bytes() const {
     return ptr.bytes() + idx.bytes() + ptr_p.bytes() + idx_p.bytes() + mask.bytes() + pos.bytes() + cell_u.bytes() + cell_p.bytes() +
-           cell_mask.bytes() + cell_h[0].bytes() + cell_h[1].bytes() + buf[0].bytes() + buf[1].bytes();
+           cell_mask.bytes() + cell_h[0].bytes() + cell_h[1].bytes();
   }
   int64_t main_values() const;  // values of the main part of buf
 };

@@ -34,7 +34,7 @@ size_t OpLevel::bytes() const {
              hang_dof.bytes() + hang_ptr.bytes() + hang_src.bytes() + pres.bytes() + tnodes.bytes() +
              tpnodes.bytes();
   if (gather) b += gather->bytes();
-  for (int i = 0; i < 2; ++i) b += rows[i].bytes() + hcell[i].bytes() + frozen[i].bytes() + hang_w[i].bytes() + dinv[i].bytes();
+  for (int i = 0; i < 2; ++i) b += hcell[i].bytes() + frozen[i].bytes() + hang_w[i].bytes() + dinv[i].bytes();
   return b;
 }
 
@@ -200,11 +200,13 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
     L.frozen[1] = lv.frozen[1].get();
     if (ph.precompute_frozen && ns_lines(L)) {
       // uniform 3D levels: the layout of ns_lines.cuh, and the rows through which a product is summed
-      for (int prec = 0; prec < 2; ++prec) {
+      // (without a scratch for them the state is interpolated in every product)
+      for (int prec = 0; prec < 2 && lv.scratch; ++prec) {
         L.lc[prec] = ns_cells_per_block(k, prec, (int64_t)nc);
         L.warps[prec] = 1;  // of the general kernel (residual, diagonal, set-up): spread over the chip
+        lv.scratch->tables += ns_fq_bytes(L, prec);
         lv.fq[prec].alloc(bud, ns_fq_bytes(L, prec));
-        lv.rows[prec].alloc(bud, ns_rows_bytes(L, prec));
+        lv.scratch->reserve(ns_rows_bytes(L, prec));
         // spare slots of the last block hold zeros; the tails that no block writes are not read
         MFNS_CUDA(cudaMemset(lv.fq[prec].get(), 0, ns_fq_bytes(L, prec)));
         L.lq[prec] = lv.fq[prec].get();
@@ -279,7 +281,7 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
     for (int32_t i : lv.constrained_host) km[(size_t)i >> 5] |= 1u << (i & 31);
     lv.keep_mask = upload(bud, km);
   }
-  if (op != OP_VMASS && !lv.L.lq[0])
+  if (op != OP_VMASS && !lv.L.lq[0] && lv.scratch)
     for (int prec = 0; prec < 2; ++prec) {
       lv.deferred[prec] = gather_fits(lv) && (tensor_cells(lv.L) || !lv.L.structured || defer_uniform(lv, prec));
       if (lv.deferred[prec]) ensure_gather(lv, prec, bud);
@@ -316,6 +318,7 @@ void ensure_gather(OpLevel& lv, int prec, Budget* bud) {
   if (!lv.gather) {
     auto G = std::make_unique<NodeGather>();
     G->nu = lv.NU;
+    G->scratch = lv.scratch;
     G->n_main = lv.nu.n_nodes;
     G->slots = (int64_t)nc * lv.nu.nb;
     if (th) {
@@ -335,6 +338,9 @@ void ensure_gather(OpLevel& lv, int prec, Budget* bud) {
         }
       return v;
     };
+    const int64_t places_all = G->slots + G->slots_p;
+    lv.scratch->tables += (size_t)((places_all + G->n_main + G->n_p) * 4 + G->n_main + G->n_p) +
+                          (G->tensor ? (size_t)(places_all * 4) + nc * 20 : 0);
     G->cell_stride = G->tensor ? 1 : lv.nu.nb;
     G->slot_stride = G->tensor ? (int64_t)nc : 1;
     if (G->tensor) {
@@ -364,23 +370,22 @@ void ensure_gather(OpLevel& lv, int prec, Budget* bud) {
     G->mask = upload(bud, mask);
     lv.gather = std::move(G);
   }
-  NodeGather& G = *lv.gather;
-  if (!G.buf[prec].get()) G.buf[prec].alloc(bud, (size_t)(G.main_values() + G.slots_p) * esize(prec));
+  lv.scratch->reserve((size_t)(lv.gather->main_values() + lv.gather->slots_p) * esize(prec));
 }
 
 // a product whose node pass applies what follows it (timed: both launches; the cell launch records itself)
 static void node_product(const OpLevel& lv, int prec, const NsAfterArgs& a, cudaStream_t s) {
   const NodeGather* G = lv.L.lq[prec] ? nullptr : lv.gather.get();
   if (!G)
-    ns_cells(lv.L, prec, a.src, lv.rows[prec].get(), s);
+    ns_cells(lv.L, prec, a.src, lv.scratch->get(), s);
   else if (G->tensor)
     tensor_product(lv.L, *G, prec, a.src, s);
   else
-    op_apply_deferred(lv.L, prec, a.src, G->buf[prec].get(), G->main_values(), s);
+    op_apply_deferred(lv.L, prec, a.src, G->scratch->get(), G->main_values(), s);
   const bool timed = lv.L.timer && lv.L.timer->enabled;
   if (timed) lv.L.timer->record_pair_begin(s);
   if (!G)
-    ns_nodes(lv.L, prec, a, lv.rows[prec].get(), s);
+    ns_nodes(lv.L, prec, a, lv.scratch->get(), s);
   else
     gather_nodes(*G, prec, a, s);
   if (timed) lv.L.timer->record_pair_end(s);
@@ -483,7 +488,7 @@ void oplevel_residual_fused(const OpLevel& lv, int prec, const void* x, const vo
 
 void oplevel_diag(const OpLevel& lv, int prec, void* diag, cudaStream_t s) {
   if (lv.hp) return hp_diag(lv, prec, diag, s);
-  if (lv.L.lq[prec]) return ns_diagonal(lv.L, prec, diag, lv.rows[prec].get(), s);
+  if (lv.L.lq[prec]) return ns_diagonal(lv.L, prec, diag, lv.scratch->get(), s);
   MFNS_CUDA(cudaMemsetAsync(diag, 0, lv.n_dofs * esize(prec), s));
   op_apply(lv.L, prec, nullptr, diag, true, s);
   const int64_t nc = (int64_t)lv.constrained_host.size();

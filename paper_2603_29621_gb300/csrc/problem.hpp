@@ -41,7 +41,7 @@ struct OpLevel {
   DevBuf keep_mask;                     // uniform meshes: bitmask of the identity rows (see oplevel_vmult)
   std::unique_ptr<NodeGather> gather;   // deferred products (and restrictions into this level)
   bool deferred[2] = {false, false};    // products are deferred (FP64 / FP32)
-  DevBuf rows[2];                       // uniform 3D stabilised levels: rows of a product (ns_lines.hpp)
+  ScratchPtr scratch;                   // set before the level is built; null: products colour by colour
   int64_t n_hang = 0;
   DevBuf hang_dof, hang_ptr, hang_src, hang_w[2];
   std::vector<int32_t> pres_host;
@@ -254,7 +254,7 @@ struct Problem {
   std::vector<Workspace> ws[2];
   // FGMRES / Krylov (fp64)
   DevBuf V, Z, w, tmp, hvec, yvec, part, ptrV, ptrZ, scal;
-  DevBuf sys_r, sys_z;                  // fp64 system-size temporaries
+  DevBuf sys_r;                         // projected right-hand side (fp64)
   DevBuf mg_b32, mg_x32;                // fp32 copies for the mixed-precision preconditioner
   DevBuf cg_r, cg_z, cg_p, cg_q, cg_x;  // Stokes Schur CG (mg precision)
   DevBuf stokes_u_rhs, stokes_u_sol;    // Stokes A-block rhs/solution (mg precision)
@@ -263,7 +263,7 @@ struct Problem {
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t pc_graph = nullptr;
   cudaGraphExec_t vc_graph[2] = {nullptr, nullptr};
-  DevBuf pc_in, pc_out, vc_in[2], vc_out[2];
+  DevBuf pc_in, pc_out;
   Krylov kry;
   double* hh_host = nullptr;            // pinned: Gram--Schmidt coefficients of the last step
   // Newton / BDF (stabilised NS; allocated on first use): explicit field, residual, increment
@@ -310,11 +310,11 @@ OpLevel& mg_level(Problem& p, int i);
 // kind 1: the vector Laplacian; kind 0: Taylor--Hood Stokes (system and pressure mass on hp spaces,
 // the A block on the hp hierarchy)
 std::unique_ptr<Problem> build_problem_hp(const Forest& f, const std::vector<int32_t>& degree, const Physics& ph,
-                                          int coarse_stop_n, Budget* bud, int kind = 1);
+                                          int coarse_stop_n, Budget* bud, ScratchPtr scratch, int kind = 1);
 // hierarchy: 0 global coarsening, 1 local smoothing (vector Laplacian and the Stokes A block on a
 // locally refined mesh; an unrefined mesh needs none and gets global coarsening)
 std::unique_ptr<Problem> build_problem(const Forest& f, int kind, int k, const Physics& ph, int mg_order,
-                                       int coarse_stop_n, Budget* bud, int hierarchy = 0);
+                                       int coarse_stop_n, Budget* bud, ScratchPtr scratch, int hierarchy = 0);
 // the level workspaces alone (r, d, t, b, x per level and precision)
 void alloc_level_workspaces(Problem& p);
 

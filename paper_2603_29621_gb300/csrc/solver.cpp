@@ -56,7 +56,7 @@ static void build_local_smoothing(Problem& p, const Forest& f, int k, const Phys
                                   int coarse_stop_n, Budget* bud);
 
 std::unique_ptr<Problem> build_problem(const Forest& f, int kind, int k, const Physics& ph, int mg_order,
-                                       int coarse_stop_n, Budget* bud, int hierarchy) {
+                                       int coarse_stop_n, Budget* bud, ScratchPtr scratch, int hierarchy) {
   auto p = std::make_unique<Problem>();
   p->uid = ++g_problem_uid;
   p->kind = kind;
@@ -87,6 +87,7 @@ std::unique_ptr<Problem> build_problem(const Forest& f, int kind, int k, const P
   if (seq.size() > 32) throw Error(kErrUnsupported, "more than 32 multigrid levels");
   for (auto& s : seq) {
     auto lv = std::make_unique<OpLevel>();
+    lv->scratch = scratch;
     build_oplevel(*lv, s.first, mop, s.second, ph, bud);
     p->levels.push_back(std::move(lv));
   }
@@ -97,8 +98,10 @@ std::unique_ptr<Problem> build_problem(const Forest& f, int kind, int k, const P
   }
   if (kind == 0) {
     p->system = std::make_unique<OpLevel>();
+    p->system->scratch = scratch;
     build_oplevel(*p->system, f, OP_STOKES, k, ph, bud);
     p->pmass = std::make_unique<OpLevel>();
+    p->pmass->scratch = scratch;
     build_oplevel(*p->pmass, f, OP_PMASS, k - 1, ph, bud);
   }
   if (local) build_local_smoothing(*p, f, k, ph, mg_order, coarse_stop_n, bud);
@@ -122,7 +125,7 @@ static void build_local_smoothing(Problem& p, const Forest& f, int k, const Phys
   // level 0 and below: the base mesh with its own global-coarsening hierarchy (vector Laplacian)
   Forest base = forest_uniform(f.dim, f.n);
   const int mop = fine.op;  // OP_STOKES_A (vector Laplacian, Stokes A block) or OP_STAB_NS
-  S->base = build_problem(base, mop == OP_STAB_NS ? 2 : 1, k, ph, mg_order, coarse_stop_n, bud, 0);
+  S->base = build_problem(base, mop == OP_STAB_NS ? 2 : 1, k, ph, mg_order, coarse_stop_n, bud, fine.scratch, 0);
   std::vector<int32_t> owner(fine.nu.n_nodes, -1);
   std::vector<int32_t> cf, cl;
   {
@@ -137,8 +140,10 @@ static void build_local_smoothing(Problem& p, const Forest& f, int k, const Phys
     auto lv = std::make_unique<LsLevel>();
     const Forest lf = forest_level(f, l);
     lv->op = std::make_unique<OpLevel>();
+    lv->op->scratch = fine.scratch;
     build_oplevel(*lv->op, lf, mop, k, ph, bud, true);
     lv->full = std::make_unique<OpLevel>();
+    lv->full->scratch = fine.scratch;
     build_oplevel(*lv->full, lf, mop, k, ph, bud, false);
     if (lv->op->n_dofs != lv->full->n_dofs || lv->op->perm != lv->full->perm)
       throw Error(kErrArg, "local smoothing: level operators disagree on the numbering");
@@ -180,13 +185,13 @@ static void build_local_smoothing(Problem& p, const Forest& f, int k, const Phys
 }
 
 std::unique_ptr<Problem> build_problem_hp(const Forest& f, const std::vector<int32_t>& degree, const Physics& ph,
-                                          int coarse_stop_n, Budget* bud, int kind) {
+                                          int coarse_stop_n, Budget* bud, ScratchPtr scratch, int kind) {
   if (degree.size() != f.n_cells()) throw Error(kErrArg, "one degree per cell expected");
   if (kind != 0 && kind != 1) throw Error(kErrUnsupported, "hp problems: Stokes or its A block");
   auto uniform = [](const std::vector<int32_t>& d) {
     return std::all_of(d.begin(), d.end(), [&](int32_t k) { return k == d[0]; });
   };
-  if (uniform(degree)) return build_problem(f, kind, degree[0], ph, 1, coarse_stop_n, bud, 0);
+  if (uniform(degree)) return build_problem(f, kind, degree[0], ph, 1, coarse_stop_n, bud, scratch, 0);
   auto p = std::make_unique<Problem>();
   p->uid = ++g_problem_uid;
   p->kind = kind;
@@ -204,6 +209,7 @@ std::unique_ptr<Problem> build_problem_hp(const Forest& f, const std::vector<int
   }
   for (int kk = d[0]; kk >= 1; --kk) {  // (all linear after the loop; kept general)
     auto lv = std::make_unique<OpLevel>();
+    lv->scratch = scratch;
     build_oplevel(*lv, f, OP_STOKES_A, kk, ph, bud);
     p->levels.push_back(std::move(lv));
   }
@@ -212,6 +218,7 @@ std::unique_ptr<Problem> build_problem_hp(const Forest& f, const std::vector<int
   while (forest_can_coarsen(fc, coarse_stop_n)) {
     fc = forest_coarsen(fc);
     auto lv = std::make_unique<OpLevel>();
+    lv->scratch = scratch;
     build_oplevel(*lv, fc, OP_STOKES_A, 1, ph, bud);
     p->levels.push_back(std::move(lv));
   }
@@ -300,7 +307,6 @@ void alloc_workspaces(Problem& p) {
   p.w.alloc(bud, n * 8);
   p.tmp.alloc(bud, n * 8);
   p.sys_r.alloc(bud, n * 8);
-  p.sys_z.alloc(bud, n * 8);
   p.hvec.alloc(bud, (2 * kMaxDots + 1) * 8);
   p.yvec.alloc(bud, kMaxDots * 8);
   p.part.alloc(bud, (size_t)kRedScratch * 8);
@@ -316,10 +322,6 @@ void alloc_workspaces(Problem& p) {
   p.mg_x32.alloc(bud, n * 4);
   p.pc_in.alloc(bud, n * 8);
   p.pc_out.alloc(bud, n * 8);
-  for (int prec = 0; prec < 2; ++prec) {
-    p.vc_in[prec].alloc(bud, p.levels[0]->n_dofs * esize(prec));
-    p.vc_out[prec].alloc(bud, p.levels[0]->n_dofs * esize(prec));
-  }
   if (p.kind == 0) {
     const int64_t np = p.pmass->n_dofs;
     const size_t es = 8;  // the Stokes preconditioner keeps fp64 and fp32 copies in separate buffers
@@ -933,22 +935,22 @@ void invalidate_graphs(Problem& p) {
 }
 
 void vcycle_graph(Problem& p, int prec, const void* b, void* x, cudaStream_t s) {
+  // the level's own right-hand side and iterate, which no cycle uses on the finest level
   Workspace& w = p.ws[prec][0];
   const size_t bytes = p.levels[0]->n_dofs * esize(prec);
   if (!p.vc_graph[prec]) {
     if (!p.cap_stream) MFNS_CUDA(cudaStreamCreateWithFlags(&p.cap_stream, cudaStreamNonBlocking));
     TimerPause pause(p);
     MFNS_CUDA(cudaStreamBeginCapture(p.cap_stream, cudaStreamCaptureModeThreadLocal));
-    vcycle(p, prec, p.vc_in[prec].get(), p.vc_out[prec].get(), p.cap_stream);
+    vcycle(p, prec, w.b.get(), w.x.get(), p.cap_stream);
     cudaGraph_t g;
     MFNS_CUDA(cudaStreamEndCapture(p.cap_stream, &g));
     MFNS_CUDA(cudaGraphInstantiate(&p.vc_graph[prec], g, 0));
     MFNS_CUDA(cudaGraphDestroy(g));
   }
-  (void)w;
-  MFNS_CUDA(cudaMemcpyAsync(p.vc_in[prec].get(), b, bytes, cudaMemcpyDeviceToDevice, s));
+  MFNS_CUDA(cudaMemcpyAsync(w.b.get(), b, bytes, cudaMemcpyDeviceToDevice, s));
   MFNS_CUDA(cudaGraphLaunch(p.vc_graph[prec], s));
-  MFNS_CUDA(cudaMemcpyAsync(x, p.vc_out[prec].get(), bytes, cudaMemcpyDeviceToDevice, s));
+  MFNS_CUDA(cudaMemcpyAsync(x, w.x.get(), bytes, cudaMemcpyDeviceToDevice, s));
 }
 
 static void precondition_body(Problem& p, const double* v, double* z, cudaStream_t s) {

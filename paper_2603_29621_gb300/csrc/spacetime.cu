@@ -274,7 +274,7 @@ static void st_vmult(mfns_spacetime& st, int prec, const void* x, void* y, cudaS
 }
 
 // the P^disc space of one level: velocity block, velocity mass, cell block
-static void build_pdisc_level(StmgLevel& L, const Forest& f, int k, double nu, Budget* bud) {
+static void build_pdisc_level(StmgLevel& L, const Forest& f, int k, double nu, Budget* bud, const ScratchPtr& scratch) {
   if (!f.uniform()) throw Error(kErrUnsupported, "P^disc spaces: uniform meshes only");
   if (k < 2 || k > 4) throw Error(kErrUnsupported, "P^disc spaces: velocity degree 2..4");
   Physics ph;
@@ -282,6 +282,7 @@ static void build_pdisc_level(StmgLevel& L, const Forest& f, int k, double nu, B
   ph.div_sign = -1.0;
   L.kind = 1;
   L.A = std::make_unique<OpLevel>();
+  L.A->scratch = scratch;
   build_oplevel(*L.A, f, OP_STOKES_A, k, ph, bud);
   L.M = std::make_unique<OpLevel>();
   build_oplevel(*L.M, f, OP_VMASS, k, ph, bud);
@@ -705,7 +706,8 @@ static int stmg_fgmres(mfns_spacetime& st, const double* b, double* x, double to
   return it;
 }
 
-static void build_stmg(mfns_spacetime& st, int nu_s, double omega, int coarse_n, int inv_prec, cudaStream_t s) {
+static void build_stmg(mfns_spacetime& st, int nu_s, double omega, int coarse_n, int inv_prec,
+                       const ScratchPtr& scratch, cudaStream_t s) {
   const bool pd = st.top != nullptr;  // P^disc slab (else Taylor--Hood on st.problem)
   Budget* bud = st.bud;
   const OpLevel& A0 = pd ? *st.top->A : *st.problem->p->system;
@@ -736,9 +738,10 @@ static void build_stmg(mfns_spacetime& st, int nu_s, double omega, int coarse_n,
     std::string err;
     if (!temporal_matrices(sp.r, L->T, &err)) throw Error(kErrArg, err);
     if (pd) {
-      build_pdisc_level(*L, fs[sp.forest], sp.k, st.nu, bud);
+      build_pdisc_level(*L, fs[sp.forest], sp.k, st.nu, bud, scratch);
     } else {
       L->A = std::make_unique<OpLevel>();
+      L->A->scratch = scratch;
       build_oplevel(*L->A, fs[sp.forest], OP_STOKES, sp.k, phys, bud);
       L->M = std::make_unique<OpLevel>();
       build_oplevel(*L->M, fs[sp.forest], OP_VMASS, sp.k, phys, bud);
@@ -784,6 +787,7 @@ static void build_stmg(mfns_spacetime& st, int nu_s, double omega, int coarse_n,
         for (StmgLevel* X : {&F, &C})
           if (!X->P) {
             X->P = std::make_unique<OpLevel>();
+            X->P->scratch = scratch;
             build_oplevel(*X->P, X->A->forest, OP_PMASS, X->k - 1, phys, bud);
           }
         F.tp = std::make_unique<Transfer>();
@@ -940,7 +944,9 @@ extern "C" int mfns_spacetime_mg_build(mfns_spacetime* st, int nu_s, double omeg
   if (!st || (inverse_precision != 0 && inverse_precision != 1)) return capi_fail(kErrArg, "bad arguments");
   MFNS_CUDA(cudaSetDevice(st->ctx->device));
   st->mg.reset();
-  build_stmg(*st, nu_s, omega, coarse_n, inverse_precision, reinterpret_cast<cudaStream_t>(stream));
+  build_within_budget(st->bud, [&](const ScratchPtr& scratch) {
+    build_stmg(*st, nu_s, omega, coarse_n, inverse_precision, scratch, reinterpret_cast<cudaStream_t>(stream));
+  });
   ST_END
 }
 
@@ -1051,15 +1057,17 @@ extern "C" int mfns_spacetime_create_pdisc(mfns_ctx* ctx, const mfns_mesh* mesh,
   st->tau = tau;
   std::string err;
   if (!temporal_matrices(r, st->T, &err)) return capi_fail(kErrArg, err.c_str());
-  auto L = std::make_unique<StmgLevel>();
-  L->k = k;
-  L->r = r;
-  L->Q = r + 1;
-  L->T = st->T;
-  build_pdisc_level(*L, mesh->forest, k, nu, st->bud);
-  L->vmx.alloc(st->bud, (size_t)L->Q * L->n * 8);
-  st->n = L->n;
-  st->top = std::move(L);
+  build_within_budget(st->bud, [&](const ScratchPtr& scratch) {
+    auto L = std::make_unique<StmgLevel>();
+    L->k = k;
+    L->r = r;
+    L->Q = r + 1;
+    L->T = st->T;
+    build_pdisc_level(*L, mesh->forest, k, nu, st->bud, scratch);
+    L->vmx.alloc(st->bud, (size_t)L->Q * L->n * 8);
+    st->n = L->n;
+    st->top = std::move(L);
+  });
   *out = st.release();
   ST_END
 }

@@ -744,7 +744,7 @@ static void launch(const OpLaunch& L, const NodeGather& g, int prec, const void*
       for (int i = 0; i < NP; ++i)
         for (int m = 0; m < NP; ++m) a.tab.Pp[hf][i][m] = (T)L.Pp[(hf * NP + i) * NP + m];
   a.src = static_cast<const T*>(src);
-  a.buf = g.buf[prec].as<T>();
+  a.buf = static_cast<T*>(g.scratch->get());
   a.buf_p = a.buf + g.main_values();
   a.cu = g.cell_u.as<int32_t>();
   a.cp = g.cell_p.as<int32_t>();

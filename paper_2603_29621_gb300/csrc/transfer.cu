@@ -330,7 +330,8 @@ void build_transfer(Transfer& t, const OpLevel& fine, const OpLevel& coarse, Bud
     }
   const_cast<OpLevel&>(fine).tnodes = upload(bud, fn);
   // restriction: contributions of every coarse cell in one launch, gathered per coarse node
-  for (int prec = 0; prec < 2 && gather_fits(coarse); ++prec) ensure_gather(const_cast<OpLevel&>(coarse), prec, bud);
+  if (coarse.scratch && gather_fits(coarse))
+    for (int prec = 0; prec < 2; ++prec) ensure_gather(const_cast<OpLevel&>(coarse), prec, bud);
   // 1D matrices
   std::vector<double> xf = gll_nodes(fine.k), xc = gll_nodes(coarse.k);
   t.E.assign(2 * NF * NC, 0.0);
@@ -374,7 +375,7 @@ static void launch_transfer(const Transfer& t, const OpLevel& fine, const OpLeve
     return;
   }
   if (coarse.gather) {  // every coarse cell in one launch; transfer_restrict gathers
-    a.defer = coarse.gather->buf[sizeof(T) == 8 ? 0 : 1].template as<T>();
+    a.defer = static_cast<T*>(coarse.gather->scratch->get());
     a.pos = coarse.gather->pos.template as<int32_t>();
     a.cell_stride = coarse.gather->cell_stride;
     a.slot_stride = coarse.gather->slot_stride;
