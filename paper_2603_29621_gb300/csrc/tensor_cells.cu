@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
     __syncthreads();
   }
   // ---- x
-  for (int it = threadIdx.x; it < vel; it += 256) {
+  for (int it = threadIdx.x; it < vel; it += TH) {
     const int c = it / (COMP * NL), f = it / NL % COMP, w = it % NL;
     T* A = mem + c * CELL + f * NB;
     T v[N];
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
     }
   }
   if constexpr (KIND == 1)
-    for (int it = threadIdx.x; it < ncell * NPL; it += 256) {
+    for (int it = threadIdx.x; it < ncell * NPL; it += TH) {
       const int c = it / NPL, w = it % NPL;
       T* cell = mem + c * CELL;
       T v[NP];
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
     }
   __syncthreads();
   // ---- y
-  for (int it = threadIdx.x; it < vel; it += 256) {
+  for (int it = threadIdx.x; it < vel; it += TH) {
     const int c = it / (COMP * NL), f = it / NL % COMP, w = it % NL;
     T* A = mem + c * CELL + f * NB + w % N + NL * (w / N);
     T v[N], z[N];
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
     }
   }
   if constexpr (KIND == 1) {
-    for (int it = threadIdx.x; it < ncell * NP * N; it += 256) {  // divergence, lines (m, z)
+    for (int it = threadIdx.x; it < ncell * NP * N; it += TH) {  // divergence, lines (m, z)
       const int c = it / (NP * N), w = it % (NP * N), m = w % NP, zc = w / NP;
       const T* W = mem + c * CELL + Tl::oW + zc * N * NP + m;
       T* t = mem + c * CELL + Tl::oT + zc * NPL + m;
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
         t[NPL * N + NP * j] = row_dot<NP, N, true>(a.tab.Mr, j, v2);
       }
     }
-    for (int it = threadIdx.x; it < ncell * N * NP; it += 256) {  // pressure, lines (x, k)
+    for (int it = threadIdx.x; it < ncell * N * NP; it += TH) {  // pressure, lines (x, k)
       const int c = it / (N * NP), w = it % (N * NP), x = w % N, kz = w / N;
       const T* q = mem + c * CELL + Tl::oP + kz * NP * N + x;
       T* o = mem + c * CELL + Tl::oPP + kz * NL + x;
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
   }
   __syncthreads();
   // ---- z, and the output where nothing hangs
-  for (int it = threadIdx.x; it < vel; it += 256) {
+  for (int it = threadIdx.x; it < vel; it += TH) {
     const int c = it / (COMP * NL), f = it / NL % COMP, w = it % NL;
     T* A = mem + c * CELL + f * NB + w;
     const T h = a.h[c0 + c];
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
     }
   }
   if constexpr (KIND == 1)
-    for (int it = threadIdx.x; it < ncell * NPL; it += 256) {
+    for (int it = threadIdx.x; it < ncell * NPL; it += TH) {
       const int c = it / NPL, w = it % NPL;
       const T* t = mem + c * CELL + Tl::oT + w;
       const T h = a.h[c0 + c];
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
   if (!any) return;
   for (int dir = 1; dir >= 0; --dir) {  // the remaining transposed interpolations, then the output
     __syncthreads();
-    for (int it = threadIdx.x; it < vel; it += 256) {
+    for (int it = threadIdx.x; it < vel; it += TH) {
       const int c = it / (COMP * NL), f = it / NL % COMP, w = it % NL;
       const uint32_t m = a.mask[c0 + c];
       int p0, st;
@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(TH, 768 / TH) k_tensor_lines(const __grid_cons
       }
     }
     if constexpr (KIND == 1)
-      for (int it = threadIdx.x; it < ncell * NPL; it += 256) {
+      for (int it = threadIdx.x; it < ncell * NPL; it += TH) {
         const int c = it / NPL, w = it % NPL;
         const uint32_t m = a.mask[c0 + c];
         int p0, st;

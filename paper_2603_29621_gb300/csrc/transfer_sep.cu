@@ -94,7 +94,6 @@ struct TensorArgs {
   const int32_t *lo, *hi;    // first / last input node of the rows >= r / <= r
   int Mi, Mo, dim, nvel;
   int rows, cols, xblocks;   // output tile of a block, blocks along x
-  int width;                 // entries of the longest row
   // first smoothing step of the coarse level from a zero iterate: x = d = c2 dinv out (x null: none)
   T *x, *d;
   const T* dinv;
@@ -377,7 +376,6 @@ static void sep_apply(const SepTransfer& t, const SepDir& d, int64_t Mi, int64_t
   a.rows = d.rows[prec];
   a.cols = d.cols[prec];
   a.xblocks = (int)((Mo + a.cols - 1) / a.cols);
-  a.width = d.width;
   if (st) {
     a.x = static_cast<T*>(st->x);
     a.d = static_cast<T*>(st->d);
