@@ -5,6 +5,7 @@
 #include <numeric>
 #include <unordered_map>
 
+#include "gather_table.hpp"
 #include "ns_lines.hpp"
 #include "problem.hpp"
 #include "tensor_cells.hpp"
@@ -296,17 +297,6 @@ void build_oplevel(OpLevel& lv, const Forest& f, int op, int k, const Physics& p
   lv.pres = upload(bud, lv.pres_host);
 }
 
-// node tables: nodes[e] is the node of place e (bit 31 ignored)
-static void gather_table(const std::vector<int32_t>& nodes, int64_t n, std::vector<int32_t>& ptr,
-                         std::vector<int32_t>& idx) {
-  ptr.assign((size_t)n + 1, 0);
-  for (int32_t g : nodes) ++ptr[(size_t)(g & 0x7fffffff) + 1];
-  for (int64_t g = 0; g < n; ++g) ptr[g + 1] += ptr[g];
-  idx.resize(nodes.size());
-  std::vector<int32_t> at(ptr.begin(), ptr.end() - 1);
-  for (size_t e = 0; e < nodes.size(); ++e) idx[at[nodes[e] & 0x7fffffff]++] = (int32_t)e;
-}
-
 bool gather_fits(const OpLevel& lv) {
   return !lv.hp && (int64_t)lv.L.n_cells * lv.nu.nb * (lv.NU == 3 ? 4 : lv.NU) <= kDeferMaxValues;
 }
@@ -328,14 +318,10 @@ void ensure_gather(OpLevel& lv, int prec, Budget* bud) {
     G->tensor = tensor_cells(lv.L);
     std::vector<int32_t> ptr, idx;
     auto places = [&](const NodeSpace& sp, bool flag) {  // masters by place
-      std::vector<int32_t> v(nc * sp.nb);
-      for (size_t i = 0; i < nc; ++i)
-        for (int b = 0; b < sp.nb; ++b) {
-          const size_t c = G->tensor ? i : (size_t)lv.perm[i];
-          int32_t g = sp.cell_master[c * sp.nb + b];
-          if (flag && lv.op != OP_PMASS && sp.boundary[g]) g |= int32_t(0x80000000u);
-          v[G->tensor ? (size_t)b * nc + i : i * sp.nb + b] = g;
-        }
+      std::vector<int32_t> v = nodes_by_place(sp.cell_master, sp.nb, lv.perm, G->tensor);
+      if (flag && lv.op != OP_PMASS)
+        for (int32_t& g : v)
+          if (sp.boundary[g]) g |= int32_t(0x80000000u);
       return v;
     };
     const int64_t places_all = G->slots + G->slots_p;
