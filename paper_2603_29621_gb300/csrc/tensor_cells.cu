@@ -712,13 +712,11 @@ static const Integrals& integrals(int k) {
   return all[k];
 }
 
+// the tables of a kernel, but for the hanging-node interpolation
 template <int N, int NP, int KIND, typename T>
-static void launch(const OpLaunch& L, const NodeGather& g, int prec, const void* src, cudaStream_t s) {
-  TpArgs<T, N, NP> a{};
+static TpTab<T, N, NP> make_tables() {
+  TpTab<T, N, NP> tab{};
   const Integrals& I = integrals(N - 1);
-  for (int hf = 0; hf < 2; ++hf)
-    for (int i = 0; i < N; ++i)
-      for (int j = 0; j < N; ++j) a.tab.P[hf][i][j] = (T)L.P[(hf * N + i) * N + j];
   auto fold = [](const long double (&x)[5][5], auto& t) {
     constexpr int H = N / 2;
     for (int i = 0; i < H; ++i) {
@@ -731,14 +729,26 @@ static void launch(const OpLaunch& L, const NodeGather& g, int prec, const void*
     }
     t.mid = (T)x[H][H];
   };
-  fold(I.m, a.tab.M);
-  fold(I.k, a.tab.K);
+  fold(I.m, tab.M);
+  fold(I.k, tab.K);
   if (KIND == 1)
     for (int i = 0; i < N; ++i)
       for (int m = 0; m < NP; ++m) {
-        a.tab.Mr[i][m] = (T)I.mr[i][m];
-        a.tab.Dr[i][m] = (T)I.dr[i][m];
+        tab.Mr[i][m] = (T)I.mr[i][m];
+        tab.Dr[i][m] = (T)I.dr[i][m];
       }
+  return tab;
+}
+
+template <int N, int NP, int KIND, typename T>
+static void launch(const OpLaunch& L, const NodeGather& g, int prec, const void* src, cudaStream_t s) {
+  // (formed once: extended precision is software on Arm, 1 to 2 us of a call's 11)
+  static const TpTab<T, N, NP> tables = make_tables<N, NP, KIND, T>();
+  TpArgs<T, N, NP> a{};
+  a.tab = tables;
+  for (int hf = 0; hf < 2; ++hf)
+    for (int i = 0; i < N; ++i)
+      for (int j = 0; j < N; ++j) a.tab.P[hf][i][j] = (T)L.P[(hf * N + i) * N + j];
   if (KIND == 1)
     for (int hf = 0; hf < 2; ++hf)
       for (int i = 0; i < NP; ++i)
