@@ -154,7 +154,7 @@ def kernel_src_hash():
 
 
 def ncu_traffic():
-    """DRAM bytes per launch of the FP32 cell kernel from the committed ncu summary,
+    """DRAM bytes of one FP32 product (both launches) from the committed ncu summary,
     or None when the kernel sources changed since the capture."""
     path = os.path.join(ROOT, "profiles", "ns_product_q2_fp32.md")
     if not os.path.exists(path):
@@ -167,7 +167,7 @@ def ncu_traffic():
     if vals.get("kernel_source_sha256_16") != kernel_src_hash():
         return None
     try:
-        return float(vals["dram_bytes_per_full_launch"])
+        return float(vals["dram_bytes_per_product"])
     except (KeyError, ValueError):
         return None
 

@@ -147,7 +147,9 @@ static void set_smem(Kern kern, size_t bytes, std::atomic<uint64_t>& done) {
 
 // Shared memory of a cell launch, raised so that no SM takes more than its share of a grid that does not
 // fill the chip: a dependent launch finds some SMs free before others, and its blocks would pile up
-// there (V-cycles FP32 48^3 1115 -> 1086 us, 8^3 181 -> 173 us).
+// there (V-cycles FP32 48^3 1115 -> 1086 us, 8^3 181 -> 173 us).  It keeps other streams' blocks off those
+// SMs for as long as the launch lasts; problems on streams of their own are still faster than with colour launches
+// (8 V-cycles of Q2 8^3 at a time, each: 61 -> 40 us, of 20^3 176 -> 116, of Q3 8^3 92 -> 87 us).
 static size_t spread_smem(size_t need, int64_t blocks) {
   const int64_t per_sm = (blocks + 151) / 152;
   if (per_sm > 16) return need;

@@ -23,7 +23,7 @@
 // and for several in a launch.
 //
 // Measured against eight colour launches of the warp-per-three-cells kernel (whole product, GB300): Q2
-// 64^3 FP32 176 -> 119 us, 48^3 FP64 1849 -> 1116 us (FP64 pipe 87 % busy), Q3 31^3 FP32 61.8 -> 58 us,
+// 64^3 FP32 176 -> 119 us, 48^3 FP64 1849 -> 1116 us (FP64 pipe 87 % busy), Q3 31^3 FP32 61.8 -> 51 us,
 // five Q1 45^3 FP32 smoothing sweeps 116 -> 50 us.  The FP32 cell launch (95 us at 64^3) is bound by
 // the DRAM stream of the point values (5.7 TB/s), the node pass (about 25 us) by its rows.
 #pragma once

@@ -12,7 +12,7 @@ namespace mfns {
 // whether L's products take this path once its point values are laid out (L.lq, L.lc)
 bool ns_lines(const OpLaunch& L);
 int ns_cells_per_block(int k, int prec, int64_t cells);
-// bytes of the level's point values and of its row buffer (needs L.lc)
+// bytes of the level's point values and of a product's rows (needs L.lc)
 size_t ns_fq_bytes(const OpLaunch& L, int prec);
 size_t ns_rows_bytes(const OpLaunch& L, int prec);
 
@@ -48,7 +48,7 @@ struct NsAfterArgs {
 };
 void ns_nodes(const OpLaunch& L, int prec, const NsAfterArgs& a, void* rows, cudaStream_t s);
 
-// diagonal with 1 on the identity rows; rows: the level's row buffer (scratch)
+// diagonal with 1 on the identity rows; rows: the buffer of a product's rows (scratch)
 void ns_diagonal(const OpLaunch& L, int prec, void* diag, void* rows, cudaStream_t s);
 
 }  // namespace mfns
