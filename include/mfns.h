@@ -389,8 +389,9 @@ int mfns_solve_begin(mfns_problem* p, const void* b, void* x, int64_t n, void* s
 int mfns_batch_step(mfns_problem** problems, int n, int* running);
 /* One V-cycle (zero initial guess) for each of n problems of one context, batched: the
  * operator applications of all problems whose current multigrid levels share dimension, degree,
- * operator, precision and smoother run as one launch per level and colour over the cells of all
- * of them, each block reading its problem from a descriptor table (uneven sizes share launches).
+ * operator, precision, smoother and kind of product run as one launch per level (and colour, where
+ * the level has those) over the cells of all of them, each block reading its problem from a
+ * descriptor table (uneven sizes share launches; 3D STOKES_A problems run their own products).
  * Results equal n separate mfns_vcycle calls (bitwise: the per-cell arithmetic and its order are
  * those of a single-problem launch).  b[i], x[i]: device vectors of problem i in `precision`, of
  * lengths[i] (host array) entries each, which must equal problem i's cycle_dofs.

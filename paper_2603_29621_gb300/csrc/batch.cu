@@ -62,8 +62,7 @@ static void fill_ns(MultiOp& m, Budget* bud) {
 template <typename T>
 static void fill(MultiOp& m, Budget* bud) {
   if (m.L0->lq[m.prec]) return fill_ns(m, bud);
-  // (a member beyond the deferred products' bound would round differently alone and in a batch)
-  if (std::all_of(m.lv.begin(), m.lv.end(), [&](const OpLevel* l) { return l->gather && l->gather->tensor; })) return;
+  if (m.lv[0]->gather && m.lv[0]->gather->tensor) return;  // tensor-product cells: the members' own products
   const OpLaunch& L0 = *m.L0;
   const int nmem = (int)m.lv.size();
   const int ncol = L0.n_colors;
@@ -122,7 +121,8 @@ MultiOp* multi_op_create(const std::vector<const OpLevel*>& lv, const std::vecto
     const OpLaunch& L = l->L;
     if (!L.structured || L.dim != L0.dim || L.k != L0.k || L.op != L0.op || L.n_colors != L0.n_colors ||
         (L.fq[prec] != nullptr) != (L0.fq[prec] != nullptr) ||
-        (L.lq[prec] != nullptr) != (L0.lq[prec] != nullptr) || L.warps[prec] != L0.warps[prec])
+        (L.lq[prec] != nullptr) != (L0.lq[prec] != nullptr) || L.warps[prec] != L0.warps[prec] ||
+        (l->gather && l->gather->tensor) != (lv[0]->gather && lv[0]->gather->tensor))
       throw Error(kErrArg, "multi-op: members differ in kind, degree, layout or block size");
   }
   auto m = std::make_unique<MultiOp>();

@@ -1330,12 +1330,15 @@ BatchVcyclePtr make_batch_vcycle(const std::vector<Problem*>& ps, int prec, cons
   B->groups.resize(B->steps);
   for (int t = 0; t < B->steps; ++t) {
     // members: problems for which level t is not the coarse level; grouped by what one launch shares
-    std::map<std::tuple<int, int, int, bool, int, int, int>, std::vector<int>> key;
+    std::map<std::tuple<int, int, int, int, int, int, int>, std::vector<int>> key;
     for (int i = 0; i < (int)ps.size(); ++i) {
       const Problem& p = *ps[i];
       if (t >= (int)p.levels.size() - 1) continue;
-      const OpLaunch& L = p.levels[t]->L;
-      key[{L.dim, L.k, L.op, L.fq[prec] || L.lq[prec], L.warps[prec], p.smoother, p.smoother_degree}].push_back(i);
+      const OpLevel& lv = *p.levels[t];
+      const OpLaunch& L = lv.L;
+      // products that round differently do not share a launch: a problem gives the same alone and in a batch
+      const int product = (L.fq[prec] ? 1 : 0) | (L.lq[prec] ? 2 : 0) | (lv.gather && lv.gather->tensor ? 4 : 0);
+      key[{L.dim, L.k, L.op, product, L.warps[prec], p.smoother, p.smoother_degree}].push_back(i);
     }
     for (auto& kv : key) {
       BatchGroup g;

@@ -53,6 +53,24 @@ def test_a_tight_budget_changes_the_layout_only(kind, dim, n, k, ball):
     assert e.value.code == L.ERR_BUDGET
 
 
+@pytest.mark.parametrize("kind,k,n", [("a", 2, 6), ("a", 3, 4), ("ns", 2, 7)])
+def test_batches_of_both_layouts(kind, k, n):
+    """A problem with the products' buffer and one without it in a batch: each gives what it gives alone, bit for
+    bit (their products round differently, so they must not share launches)."""
+    from paper_2603_29621_gb300 import _lib as L, api
+    ctx, p = _problem(0, kind, 3, n, k, 0)
+    tight = api.Context(0, hbm_budget_bytes=2 * ctx.memory()[0] - 1)
+    ps = [api.Problem(tight, api.Mesh(tight, 3, n), kind=L.STAB_NS if kind == "ns" else L.STOKES_A, degree=k, nu=0.1,
+                      dt=1e-2 if kind == "ns" else 0.0, lambda_max=2.0, mg_precision=L.FP32) for _ in range(2)]
+    assert tight.memory()[0] < 2 * ctx.memory()[0]
+    for dt in (torch.float64, torch.float32):
+        bs = [torch.tensor(inputs.uniform_vector(p.info.cycle_dofs, seed=s), device="cuda", dtype=dt) for s in (4, 5)]
+        xs = [torch.zeros_like(b) for b in bs]
+        api.batch_vcycle(ps, bs, xs)
+        for q, b, x in zip(ps, bs, xs):
+            assert torch.equal(x, q.vcycle(b, torch.zeros_like(b)))
+
+
 def test_a_refused_problem_leaves_nothing_allocated():
     from paper_2603_29621_gb300 import _lib as L, api
     ctx = api.Context(0, hbm_budget_bytes=1 << 20)
